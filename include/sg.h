@@ -117,7 +117,7 @@ typedef struct sg_options {
                                diagonal), the even cells (i + j + k) first; levels == 1
                                runs one sweep per cycle (App. B's single-level GS /
                                SOR); the coarsest level keeps the RKL1 schedule; the
-                               fused and cluster kernels are not used; periodic axes
+                               fused super-steps are not used; periodic axes
                                need even extents on the swept levels (SG_ERR_ARG
                                from sg_solve otherwise)                        [RKL]*/
     double omega;           /* GS-RB relaxation factor in [0, 2): 1 = Gauss-Seidel,
@@ -203,8 +203,8 @@ sg_status sg_create_grid(int nx, int ny, int nz, const double lo[3], const doubl
  * stages, coarsest solve and ghost rules (Sec. 2.3) as the 3D grid.  Every
  * other call takes the grid as a 3D grid with nz = 1: arrays are [1][ny][nx]
  * = [ny][nx]; faces -x, +x are [ny], -y, +y are [nx]; the z faces are unused
- * (pass NULL).  Level rule of Sec. 4.1 on x and y.  The fused super-step and
- * cluster kernels are 3D-only; a 2D grid runs the per-stage kernels.  Sizes:
+ * (pass NULL).  Level rule of Sec. 4.1 on x and y.  The fused super-step is
+ * 3D-only; the finer levels of a 2D grid run the per-stage kernels.  Sizes:
  * 2 <= n_d <= 65536, nx * ny <= 2^31 - 1.  Errors as sg_create_grid.
  */
 sg_status sg_create_grid_2d(int nx, int ny, const double lo[2], const double hi[2], const int bc[2], int precision,
@@ -399,13 +399,17 @@ sg_status sg_plan_sor_omega(int nx, int ny, int nz, const double lo[3], const do
  * microseconds per launch, so time solves with it disabled) and the totals are
  * kept per kernel class.  `bytes` is the algorithmic traffic of the launches:
  * the compulsory reads and writes of their input and output arrays, each cell
- * counted once, independent of caching.
+ * counted once, independent of caching.  While the profile is on, the cluster
+ * launch that otherwise runs every coarse level that fits it (and, for small
+ * grids, the whole solve) takes only the two coarsest levels, so that the other
+ * classes are seen at every level; results agree to FP32 rounding of the inner
+ * V-cycle.
  * ------------------------------------------------------------------------ */
 #define SG_KERNEL_CLASSES 11
 typedef struct sg_kernel_stat {
     char      name[24];       /* rkl_stage_l0, rkl_stage_coarse, residual_l0, residual_restrict,
                                  prolong_correct, coarse_solve, update, reduce_misc,
-                                 bottom_levels (the two coarsest levels in one launch),
+                                 bottom_levels (the coarse levels in one launch),
                                  gsrb_sweep (one colour of a GS-RB sweep),
                                  gravity (sg_gravity) */
     long long launches;

@@ -38,26 +38,16 @@ __global__ void k_loop_step(DeviceLoop* dl, const Reduced* red, const int* ss_do
     long long cs = 0;
     for (int q = 0; q < ss && q < d.sched_len; ++q) cs += sched[q];
     d.coarse_stage_cells += cs * d.coarse_cells;
-    d.m += 1;
-    const double rel = loop_rel(d, *red), maxabs = red->maxabs;
-    const bool finite = isfinite(rel);
-    unsigned go = 0;
-    if (!d.fixed && finite && loop_met(d, rel, maxabs) && d.confirm) {
-        d.pending = 1;                      // the true residual decides (loop_confirm)
-    } else {
-        loop_record(d, rel, maxabs);
-        if (!finite) d.status = kLoopNonFinite;
-        else if (!d.fixed && loop_met(d, rel, maxabs)) d.status = kLoopDone;
-        else if (d.m >= d.limit) d.status = d.fixed ? kLoopDone : kLoopNotConverged;
-        else go = 1;
-    }
-    cudaGraphSetConditional(inner, go);
+    bool record;
+    const bool go = loop_decide(d, loop_rel(d, *red), red->maxabs, &record);
+    if (record && d.m < kLoopHistory) d.history[d.m] = d.rel;
+    cudaGraphSetConditional(inner, go ? 1u : 0u);
 }
 
 // After the inner loop (mixed precision: the true FP64 residual is in red):
 // confirm, or resume the cycles.
 __global__ void k_loop_confirm(DeviceLoop* dl, const Reduced* red, cudaGraphConditionalHandle outer,
-                               cudaGraphConditionalHandle inner) {
+                               cudaGraphConditionalHandle inner, int has_inner) {
     DeviceLoop& d = *dl;
     unsigned go = 0;
     d.confirms += 1;
@@ -70,23 +60,24 @@ __global__ void k_loop_confirm(DeviceLoop* dl, const Reduced* red, cudaGraphCond
         else if (d.m >= d.limit) d.status = kLoopNotConverged;
         else go = 1;
     }
-    cudaGraphSetConditional(inner, go);
+    if (has_inner) cudaGraphSetConditional(inner, go);
     cudaGraphSetConditional(outer, go);
 }
 
 // Before the loop: both conditions from the state the host wrote (a solve
 // already finished at its first residual runs no cycle).
-__global__ void k_loop_init(const DeviceLoop* dl, cudaGraphConditionalHandle outer, cudaGraphConditionalHandle inner) {
+__global__ void k_loop_init(const DeviceLoop* dl, cudaGraphConditionalHandle outer, cudaGraphConditionalHandle inner,
+                            int has_inner) {
     const unsigned go = dl->status == kLoopRunning ? 1u : 0u;
     cudaGraphSetConditional(outer, go);
-    cudaGraphSetConditional(inner, go);
+    if (has_inner) cudaGraphSetConditional(inner, go);
 }
 
 }  // namespace
 
 cudaError_t launch_loop_init(const DeviceLoop* d, cudaGraphConditionalHandle outer, cudaGraphConditionalHandle inner,
-                             cudaStream_t st) {
-    k_loop_init<<<1, 1, 0, st>>>(d, outer, inner);
+                             bool has_inner, cudaStream_t st) {
+    k_loop_init<<<1, 1, 0, st>>>(d, outer, inner, has_inner ? 1 : 0);
     return cudaGetLastError();
 }
 
@@ -97,8 +88,8 @@ cudaError_t launch_loop_step(DeviceLoop* d, const Reduced* red, const int* ss_do
 }
 
 cudaError_t launch_loop_confirm(DeviceLoop* d, const Reduced* red, cudaGraphConditionalHandle outer,
-                                cudaGraphConditionalHandle inner, cudaStream_t st) {
-    k_loop_confirm<<<1, 1, 0, st>>>(d, red, outer, inner);
+                                cudaGraphConditionalHandle inner, bool has_inner, cudaStream_t st) {
+    k_loop_confirm<<<1, 1, 0, st>>>(d, red, outer, inner, has_inner ? 1 : 0);
     return cudaGetLastError();
 }
 

@@ -9,6 +9,7 @@
 // These are HBM-bandwidth-bound kernels; no tensor cores are involved.
 #include "sg_field_ops.cuh"
 #include "sg_internal.cuh"
+#include "sg_update.cuh"
 
 #include <algorithm>
 #include <cstdint>
@@ -98,33 +99,6 @@ __device__ __forceinline__ T lap_at(const T* u, const LevelGeom& g, int i, int j
     const T zm = (k > 0) ? u[idx - plane] : z_low<FACES>(u, g, i, j, idx, plane, c);
     const T zp = (k < g.nz - 1) ? u[idx + plane] : z_high<FACES>(u, g, i, j, idx, plane, c);
     return lap7(c, xm, xp, ym, yp, zm, zp, ih2x<T>(g), ih2y<T>(g), ih2z<T>(g));
-}
-
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& err) {
-    s = a + b;
-    const float bb = s - a;
-    err = (a - (s - bb)) + (b - bb);
-}
-
-// float -> double from the IEEE fields (subnormal floats, below 1.2e-38, become 0).
-__device__ __forceinline__ double f2d_bits(float x) {
-    const unsigned u = __float_as_uint(x);
-    const unsigned sgn = u & 0x80000000u, ex = (u >> 23) & 0xffu, m = u & 0x7fffffu;
-    unsigned hi, lo;
-    if (ex == 0u) { hi = sgn; lo = 0u; }
-    else if (ex == 255u) { hi = sgn | 0x7ff00000u | (m >> 3); lo = m << 29; }
-    else { hi = sgn | ((ex + 896u) << 20) | (m >> 3); lo = m << 29; }
-    return __hiloint2double((int)hi, (int)lo);
-}
-
-// double -> float by truncating the significand (within one FP32 ulp; values
-// below 2^-126 become 0, beyond the FP32 range +-inf).
-__device__ __forceinline__ float d2f_bits(double x) {
-    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-    const unsigned sgn = hi & 0x80000000u, ex = (hi >> 20) & 0x7ffu, mh = hi & 0xfffffu;
-    if (ex <= 896u) return __uint_as_float(sgn);
-    if (ex >= 1151u) return __uint_as_float(sgn | 0x7f800000u | ((ex == 2047u && (mh | lo)) ? 0x400000u : 0u));
-    return __uint_as_float(sgn | ((ex - 896u) << 23) | (mh << 3) | (lo >> 29));
 }
 
 // A residual in the output precision: FP64 -> FP32 by the bit-level
@@ -1141,45 +1115,6 @@ k_prolong_correct4(const LevelGeom g, const float* __restrict__ coarse, float* _
 // of the FP32 rate, and this kernel keeps three of them per cell (phi + e and
 // the two FMAs).
 // ---------------------------------------------------------------------------
-// r -= (A_0 e) for one cell, A_0 the homogeneous operator, formed without
-// rounding: the FP32 neighbour sum is split by TwoSum into a value and its
-// exact error (products by -6 and -2 are exact up to one FMA term), and both
-// enter r through FP64 FMAs.
-template <bool UNIFORM>
-__device__ __forceinline__ double update_r(const LevelGeom& g, float c, float xm, float xp, float ym, float yp,
-                                           float zm, float zp, double r) {
-    if (UNIFORM) {
-        // sum of the six neighbours minus 6 c, compensated
-        const float p = -6.0f * c;
-        const float perr = fmaf(-6.0f, c, -p);          // -6 c = p + perr exactly
-        float s = xm, comp = perr, t;
-        two_sum(s, xp, s, t); comp += t;
-        two_sum(s, ym, s, t); comp += t;
-        two_sum(s, yp, s, t); comp += t;
-        two_sum(s, zm, s, t); comp += t;
-        two_sum(s, zp, s, t); comp += t;
-        two_sum(s, p, s, t); comp += t;
-        const double nih2 = -g.ihx2;
-        r = fma(nih2, f2d_bits(s), r);
-        r = fma(nih2, f2d_bits(comp), r);
-    } else {
-        // per-axis second differences (-2 c is exact), compensated
-        const float m2 = -2.0f * c;
-        const float a[3][2] = {{xm, xp}, {ym, yp}, {zm, zp}};
-        const double ih[3] = {g.ihx2, g.ihy2, g.ihz2};
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            float s, comp, t;
-            two_sum(a[d][0], a[d][1], s, comp);
-            two_sum(s, m2, s, t);
-            comp += t;
-            r = fma(-ih[d], f2d_bits(s), r);
-            r = fma(-ih[d], f2d_bits(comp), r);
-        }
-    }
-    return r;
-}
-
 template <bool UNIFORM>
 __global__ void __launch_bounds__(BX * BY)
 k_update_residual(const LevelGeom g, double* __restrict__ phi, const float* __restrict__ e,
@@ -1198,7 +1133,7 @@ k_update_residual(const LevelGeom g, double* __restrict__ phi, const float* __re
             const float zp = (k < g.nz - 1) ? e[idx + plane] : z_high<false>(e, g, i, j, idx, plane, c);
             float xm, xp, ym, yp;
             xy_neighbours<false>(e, g, i, j, k, idx, c, xm, xp, ym, yp);
-            const double r = update_r<UNIFORM>(g, c, xm, xp, ym, yp, zm, zp, r64[idx]);
+            const double r = update_r<UNIFORM>(g.ihx2, g.ihy2, g.ihz2, c, xm, xp, ym, yp, zm, zp, r64[idx]);
             r64[idx] = r;
             phi[idx] = phi[idx] + f2d_bits(c);
             const float rf = d2f_bits(r);
@@ -1243,10 +1178,10 @@ k_update_residual4(const LevelGeom g, double* __restrict__ phi, const float* __r
             const float xr = i0 + 4 < nx ? e[idx + 4] : (px ? e[idx + 4 - nx] : -c.w);
             double2 ra = ld_d2(r64 + idx), rb = ld_d2(r64 + idx + 2);
             double2 pa = ld_d2(phi + idx), pb = ld_d2(phi + idx + 2);
-            ra.x = update_r<UNIFORM>(g, c.x, xl, c.y, ym.x, yp.x, zm.x, zp.x, ra.x);
-            ra.y = update_r<UNIFORM>(g, c.y, c.x, c.z, ym.y, yp.y, zm.y, zp.y, ra.y);
-            rb.x = update_r<UNIFORM>(g, c.z, c.y, c.w, ym.z, yp.z, zm.z, zp.z, rb.x);
-            rb.y = update_r<UNIFORM>(g, c.w, c.z, xr, ym.w, yp.w, zm.w, zp.w, rb.y);
+            ra.x = update_r<UNIFORM>(g.ihx2, g.ihy2, g.ihz2, c.x, xl, c.y, ym.x, yp.x, zm.x, zp.x, ra.x);
+            ra.y = update_r<UNIFORM>(g.ihx2, g.ihy2, g.ihz2, c.y, c.x, c.z, ym.y, yp.y, zm.y, zp.y, ra.y);
+            rb.x = update_r<UNIFORM>(g.ihx2, g.ihy2, g.ihz2, c.z, c.y, c.w, ym.z, yp.z, zm.z, zp.z, rb.x);
+            rb.y = update_r<UNIFORM>(g.ihx2, g.ihy2, g.ihz2, c.w, c.z, xr, ym.w, yp.w, zm.w, zp.w, rb.y);
             *reinterpret_cast<double2*>(r64 + idx) = ra;
             *reinterpret_cast<double2*>(r64 + idx + 2) = rb;
             pa.x += f2d_bits(c.x);

@@ -640,61 +640,100 @@ bool use_fused_zero(const sg_grid* g, bool faces, int l) {
            fused_supported(g->opt.rkl_order, g->opt.s_smooth) && g->lv[l].n >= kZeroFusedMinCells;
 }
 
-// The two coarsest levels B = L - 2 >= 1 and C = L - 1 of the FP32 V-cycle
-// in one cluster launch (kernels_cluster.cu): the cluster size, or 0 where the
-// level-by-level kernels run them.
-int bottom_nc(const sg_grid* g, int L, int* threads, size_t* bytes) {
-    const int B = L - 2;
-    if (g->twod || g->precision != SG_MIXED || !g->opt.fused || g->opt.smoother != SG_SMOOTH_RKL || B < 1) return 0;
-    const Level& lb = g->lv[B];
-    return bottom_plan(lb.nx, lb.ny, lb.nz, g->opt.s_smooth, threads, bytes);
-}
-
-// e_B from f_B: B's pre-smoothing, the restriction to C, C's coarse solve, the
-// prolongation to B and B's post-smoothing, with the coefficients and the
-// schedule of the level-by-level path.
-sg_status bottom_levels(sg_grid* g, int B, const float* rhs, float* u, int nc, int threads, size_t bytes) {
-    const Level& lb = g->lv[B];
-    const Level& lc = g->lv[B + 1];
-    const LevelGeom gb = geom(g, B, false), gc = geom(g, B + 1, false);
-    const int order = g->opt.rkl_order, s = g->opt.s_smooth;
+// The levels B .. L - 1 of a V-cycle in one cluster launch (kernels_cluster.cu):
+// fills the launch for first level B with the coefficients of the level-by-level
+// path; false where it does not fit.
+template <typename W>
+bool tail_params(const sg_grid* g, int L, int B, TailParams<W>& p, TailLaunch* t) {
+    const int s = g->opt.s_smooth, order = g->opt.rkl_order;
+    p = TailParams<W>{};
+    p.nl = L - B;
+    if (p.nl > kTailMaxLevels || s > kTailMaxS) return false;
     const Rkl r = make_rkl(order, s);
-    const double tau = g->opt.tau_frac * (2.0 / lambda_max(lb)) * r.tau_over_dtpar;
-    BottomParams p{};
-    p.nx = lb.nx;
-    p.ny = lb.ny;
-    p.nz = lb.nz;
-    for (int d = 0; d < 3; ++d) p.per[d] = gb.per[d];
-    p.hx = gb.ihx2f;
-    p.hy = gb.ihy2f;
-    p.hz = gb.ihz2f;
-    p.chx = gc.ihx2f;
-    p.chy = gc.ihy2f;
-    p.chz = gc.ihz2f;
     p.order = order;
     p.s = s;
-    p.n_pre = pre_count(g, B);
-    p.n_post = post_count(g, B);
-    p.tau = float(tau);
-    p.mut1 = float(r.mut[1]);
+    p.gsrb = g->opt.smoother == SG_SMOOTH_GSRB ? 1 : 0;
+    p.mut1 = W(r.mut[1]);
     for (int j = 2; j <= s; ++j) {
-        p.mu[j] = float(r.mu[j]);
-        p.nu[j] = float(r.nu[j]);
-        p.mut_tau[j] = float(r.mut[j] * tau);
-        p.c0[j] = float(r.c0[j]);
-        p.gt[j] = float(r.gt[j]);
+        p.mu[j] = W(r.mu[j]);
+        p.nu[j] = W(r.nu[j]);
+        p.mut[j] = W(r.mut[j]);
+        p.c0[j] = W(r.c0[j]);
+        p.gt[j] = W(r.gt[j]);
+    }
+    for (int i = 0; i < p.nl; ++i) {
+        const Level& lv = g->lv[B + i];
+        const LevelGeom G = geom(g, B + i, false);
+        TailLevel<W>& q = p.lv[i];
+        q.nx = lv.nx;
+        q.ny = g->twod ? 1 : lv.ny;
+        q.nz = g->twod ? lv.ny : lv.nz;
+        q.n_pre = pre_count(g, B + i);
+        q.n_post = post_count(g, B + i);
+        q.hx = ih2x<W>(G);
+        q.hy = g->twod ? W(0) : ih2y<W>(G);
+        q.hz = g->twod ? ih2y<W>(G) : ih2z<W>(G);
+        q.md = W(-2) * (q.hx + q.hy + q.hz);
+        q.tau = W(g->opt.tau_frac * (2.0 / lambda_max(lv)) * r.tau_over_dtpar);
+        q.omega = W(gsrb_omega(g, B + i));
+        for (int d = 0; d < 3; ++d) p.per[d] = G.per[d];
+        if (g->twod) p.per[2] = G.per[1];
     }
     p.remove_mean = all_periodic(g) ? 1 : 0;
     p.sched = g->d_sched;
     p.max_ss = g->opt.coarse_max_ss;
-    p.tol = float(g->opt.coarse_tol);
-    p.tau_unit = float(coarse_c(g, B + 1) * 2.0 / lambda_max(lc));
+    p.tol = W(g->opt.coarse_tol);
+    p.tau_unit = W(coarse_c(g, L - 1) * 2.0 / lambda_max(g->lv[L - 1]));
+    p.ss_done = g->d_ss;
+    return tail_plan<W>(p, g->twod, t);
+}
+
+// First level of the cluster launch, -1: none, every level by its own kernels.
+// The finest level that fits is taken: a launch per stage costs 2.5 - 3.1 us in a
+// graph whatever the level's size, a stage of the cluster launch 0.25 - 0.7 us
+// (solves with the default options: 128^3 4.22 against 3.15 ms, 1024^2 4.66 against
+// 3.04 ms).  Level 0 joins only for the error equation (FP32, e = 0 at the start, no
+// face data).
+// While a profile is taken only the two coarsest levels are run by it, so that the
+// kernel classes of the others can be told apart.
+template <typename W>
+int tail_level(const sg_grid* g, int L, TailParams<W>& p, TailLaunch* t) {
+    if (!g->opt.fused) return -1;
+    int b = std::is_same<W, float>::value ? 0 : 1;
+    if (g->prof) {
+        b = L - 2;
+        if (b < 1 || g->twod || g->precision != SG_MIXED || g->opt.smoother != SG_SMOOTH_RKL ||
+            g->lv[L - 1].nx % 4 != 0 || (long long)g->lv[b].nx * g->lv[b].ny > 1024)
+            return -1;
+    }
+    for (; b <= L - 2; ++b)
+        if (tail_params<W>(g, L, b, p, t)) return b;
+    return -1;
+}
+
+// The whole inner loop of a mixed solve in one launch: level 0 is in the cluster, and
+// so are phi and r.
+bool resident_params(const sg_grid* g, int L, double* phi, TailParams<float>& p, TailLaunch* t) {
+    if (g->precision != SG_MIXED || !g->opt.fused || g->prof || L < 2) return false;
+    if (!tail_params<float>(g, L, 0, p, t)) return false;
+    const LevelGeom G = geom(g, 0, false);
+    p.loop = g->dloop;
+    p.phi = phi;
+    p.r64 = g->r64;
+    p.rhs = (const float*)g->lv[0].rhs;
+    p.ihx2 = G.ihx2;
+    p.ihy2 = G.ihy2;
+    p.ihz2 = G.ihz2;
+    return tail_plan<float>(p, g->twod, t);
+}
+
+template <typename W>
+sg_status tail_levels(sg_grid* g, int B, TailParams<W>& p, const TailLaunch& t, const W* rhs, W* u) {
     p.rhs = rhs;
     p.u_out = u;
-    p.ss_done = g->d_ss;
     {
-        ProfScope ps(g, K_BOTTOM, 2.0 * lb.n * sizeof(float));
-        SG_CK(launch_bottom(p, nc, threads, bytes, g->st));
+        ProfScope ps(g, K_BOTTOM, 2.0 * g->lv[B].n * sizeof(W));
+        SG_CK(launch_tail<W>(p, g->twod, t, g->st));
     }
     ++g->launches;
     return SG_OK;
@@ -738,12 +777,15 @@ sg_status vcycle(sg_grid* g, int L, W* u0, const W* rhs0, bool faces, bool zero0
         if (zero_start) SG_CK(cudaMemsetAsync(cur[l], 0, g->lv[l].n * sizeof(W), g->st));   // also for count = 0
         return relax<W>(g, l, count, fc, cur[l], R(l));
     };
-    int bottom_threads = 0;
-    size_t bottom_bytes = 0;
-    const int bottom = std::is_same<W, float>::value ? bottom_nc(g, L, &bottom_threads, &bottom_bytes) : 0;
+    TailParams<W> tail;
+    TailLaunch tail_launch;
+    const int tl = tail_level<W>(g, L, tail, &tail_launch);     // the levels tl .. L - 1 in one launch (-1: none)
+    if (tl == 0 && zero0 && !faces) {
+        if (u0_final) *u0_final = u0;
+        return tail_levels<W>(g, 0, tail, tail_launch, rhs0, u0);
+    }
     SG_TRY(smooth(0, g->opt.n_pre, zero0, faces));                              // step 1
     for (int l = 1; l < L; ++l) {                                               // step 2
-        if (bottom && l == L - 1) break;        // restricted into C inside the cluster launch
         int nb = 0;
         {
             ProfScope ps(g, K_RESTRICT, (2.0 + 0.125) * g->lv[l - 1].n * sizeof(W));
@@ -757,17 +799,14 @@ sg_status vcycle(sg_grid* g, int L, W* u0, const W* rhs0, bool faces, bool zero0
             SG_CK(launch_subtract_mean<W>((W*)g->lv[l].rhs, g->lv[l].n, g->red + 1, g->st));
             g->launches += 2;
         }
-        if constexpr (std::is_same<W, float>::value) {
-            if (bottom && l == L - 2) {                                          // levels L - 2 and L - 1
-                SG_TRY(bottom_levels(g, l, R(l), cur[l], bottom, bottom_threads, bottom_bytes));
-                continue;
-            }
+        if (l == tl) {                                                          // levels tl .. L - 1
+            SG_TRY(tail_levels<W>(g, l, tail, tail_launch, R(l), cur[l]));
+            break;
         }
         if (l < L - 1) SG_TRY(smooth(l, pre_count(g, l), true, false));         // 2c + 2d-i
         else SG_TRY(coarse_solve<W>(g, l, R(l), cur[l], g->d_ss));              // 2c + 2e
     }
-    for (int l = L - 2; l >= 1; --l) {                                          // step 3
-        if (bottom && l == L - 2) continue;     // prolonged and post-smoothed in the cluster launch
+    for (int l = (tl > 0 ? tl : L - 1) - 1; l >= 1; --l) {                      // step 3
         {
             ProfScope ps(g, K_PROLONG, (2.0 + 0.125) * g->lv[l].n * sizeof(W));
             SG_CK(launch_prolong_correct<W>(geom(g, l, false), cur[l + 1], cur[l], g->st));
@@ -1012,9 +1051,6 @@ sg_status solve_begin(sg_grid* g, SolveState& S, double tol, int L, double* phi,
         const Level& Lc = g->lv[L - 1];
         const int Nc = std::max(Lc.nx, std::max(Lc.ny, Lc.nz));
         SG_TRY(ensure_sched(g, accelerated_schedule(Nc, g->opt.coarse_max_ss)));
-        int bt = 0;
-        size_t bb = 0;
-        (void)bottom_nc(g, L, &bt, &bb);          // plan the cluster launch before any capture
     }
     S.limit = g->opt.fixed_cycles > 0 ? g->opt.fixed_cycles : g->opt.max_cycles;
     S.single_c = g->opt.single_tau_frac > 0 ? g->opt.single_tau_frac : cell_tau_frac(N0);
@@ -1047,9 +1083,9 @@ sg_status solve_check(sg_grid* g, SolveState& S) {
     S.info.rel_residual = rel;
     S.info.max_residual = g->host_red[0].maxabs;
     if (!std::isfinite(rel)) {
-        const unsigned waits = g->precision == SG_MIXED ? lean_wait_failures() : 0u;
+        const unsigned waits = g->precision == SG_MIXED ? lean_wait_failures() + tail_wait_failures() : 0u;
         S.status = fail(SG_ERR_NONFINITE, waits ? "residual norm is not finite: " + std::to_string(waits) +
-                                                      " fused super-step launch(es) gave up a bounded wait"
+                                                      " launch(es) gave up a bounded wait"
                                                 : std::string("residual norm is not finite"));
         S.done = true;
     } else if (g->opt.fixed_cycles == 0 && met(rel, g->host_red[0].maxabs)) {
@@ -1157,7 +1193,6 @@ sg_status add_solve_loop(sg_grid* g, cudaGraph_t graph, int L, double* phi, cons
     cudaStream_t st = g->st;
     cudaGraphConditionalHandle ho = 0, hi = 0;
     SG_CK(cudaGraphConditionalHandleCreate(&ho, graph, 0, cudaGraphCondAssignDefault));
-    SG_CK(cudaGraphConditionalHandleCreate(&hi, graph, 0, cudaGraphCondAssignDefault));
     // appends a WHILE node after the work captured so far on st; returns its body
     auto add_while = [&](cudaGraphConditionalHandle h, cudaGraph_t* body) -> sg_status {
         cudaStreamCaptureStatus cs;
@@ -1188,21 +1223,29 @@ sg_status add_solve_loop(sg_grid* g, cudaGraph_t graph, int L, double* phi, cons
         if (e != cudaSuccess) return fail(SG_ERR_CUDA, std::string("solve graph capture: ") + cudaGetErrorString(e));
         return SG_OK;
     };
+    // the inner loop as one launch where every level fits the cluster (mixed, RKL or
+    // GS-RB): no WHILE node inside the outer one
+    TailParams<float> tail;
+    TailLaunch tail_launch;
+    const bool resident = resident_params(g, L, phi, tail, &tail_launch);
+    if (!resident) SG_CK(cudaGraphConditionalHandleCreate(&hi, graph, 0, cudaGraphCondAssignDefault));
     cudaGraph_t outer_body = nullptr, inner_body = nullptr;
     SG_TRY(capture(graph, [&]() -> sg_status {
-        SG_CK(launch_loop_init(g->dloop, ho, hi, st));
+        SG_CK(launch_loop_init(g->dloop, ho, hi, !resident, st));
         return add_while(ho, &outer_body);
     }));
     const long long before = g->launches;
     SG_TRY(capture(outer_body, [&]() -> sg_status {
-        SG_TRY(add_while(hi, &inner_body));
+        if (resident) SG_CK(launch_tail<float>(tail, g->twod, tail_launch, st));
+        else SG_TRY(add_while(hi, &inner_body));
         const long long b0 = g->launches;
         if (g->precision == SG_MIXED) SG_TRY(level0_residual(g, phi, f, faces));
-        SG_CK(launch_loop_confirm(g->dloop, g->red, ho, hi, st));
-        *per_confirm = g->launches - b0 + 1;
+        SG_CK(launch_loop_confirm(g->dloop, g->red, ho, hi, !resident, st));
+        *per_confirm = g->launches - b0 + (resident ? 2 : 1);
         return SG_OK;
     }));
-    SG_TRY(capture(inner_body, [&]() -> sg_status {
+    *per_cycle = 0;
+    if (!resident) SG_TRY(capture(inner_body, [&]() -> sg_status {
         const long long b0 = g->launches;
         SG_TRY(cycle_core(g, L, phi, f, faces));
         SG_CK(launch_loop_step(g->dloop, g->red, g->d_ss, g->d_sched, hi, st));
@@ -1244,9 +1287,9 @@ void read_device_loop(sg_grid* g, SolveState& S, const DeviceLoop& d, long long 
     S.su += (long long)(d.m - m0) * stage_updates_per_cycle(g, S.L) + d.coarse_stage_cells;
     g->launches += 1 + (long long)(d.m - m0) * per_cycle + (long long)d.confirms * per_confirm;
     if (d.status == kLoopNonFinite) {
-        const unsigned waits = g->precision == SG_MIXED ? lean_wait_failures() : 0u;
+        const unsigned waits = g->precision == SG_MIXED ? lean_wait_failures() + tail_wait_failures() : 0u;
         S.status = fail(SG_ERR_NONFINITE, waits ? "residual norm is not finite: " + std::to_string(waits) +
-                                                      " fused super-step launch(es) gave up a bounded wait"
+                                                      " launch(es) gave up a bounded wait"
                                                 : std::string("residual norm is not finite"));
     } else if (d.status == kLoopNotConverged) {
         S.status = fail(SG_ERR_NOT_CONVERGED, "max_cycles reached above the tolerance");
@@ -1478,7 +1521,7 @@ sg_status create_grid(int nx, int ny, int nz, const double lo[3], const double h
         std::lock_guard<std::mutex> lock(configure_mu);
         SG_CK(coarse_configure());
         SG_CK(fused_configure());
-        SG_CK(bottom_configure());
+        SG_CK(tail_configure());
     }
     sg_grid* g = new sg_grid();
     static std::atomic<unsigned long long> serials{0};

@@ -142,7 +142,7 @@ constexpr int kLoopHistory = 256;          // entries of the residual history ke
 constexpr int kLoopRunning = 0, kLoopDone = 1, kLoopNotConverged = 2, kLoopNonFinite = 3;
 // State of one solve's cycle loop in device memory: set by the host before
 // the solve graph is launched, read back once when it has finished.
-struct DeviceLoop {
+struct LoopState {
     double rden;            // ||L 0 - f|| (1 if zero)
     double nn;              // cells of level 0
     double tol;             // relative L2 tolerance
@@ -158,15 +158,38 @@ struct DeviceLoop {
     long long coarse_cells; // cells of the coarsest level
     long long coarse_stage_cells;   // sum over cycles of coarse cells x stages
     double rel, maxabs;     // the last recorded residual
+};
+struct DeviceLoop : LoopState {
     double history[kLoopHistory];
     int coarse_ss[kLoopHistory];
 };
+// has_inner false: the inner loop is no WHILE node (the resident solve runs it in one launch)
 cudaError_t launch_loop_init(const DeviceLoop* d, cudaGraphConditionalHandle outer, cudaGraphConditionalHandle inner,
-                             cudaStream_t st);
+                             bool has_inner, cudaStream_t st);
 cudaError_t launch_loop_step(DeviceLoop* d, const Reduced* red, const int* ss_done, const int* sched,
                              cudaGraphConditionalHandle inner, cudaStream_t st);
 cudaError_t launch_loop_confirm(DeviceLoop* d, const Reduced* red, cudaGraphConditionalHandle outer,
-                                cudaGraphConditionalHandle inner, cudaStream_t st);
+                                cudaGraphConditionalHandle inner, bool has_inner, cudaStream_t st);
+// The decision after a cycle with relative residual rel and largest residual maxabs, on
+// the counters of d: true to run another.  *record: the residual goes into the history.
+__device__ __forceinline__ bool loop_decide(LoopState& d, double rel, double maxabs, bool* record) {
+    d.m += 1;
+    const bool finite = isfinite(rel);
+    const bool met = d.mtol > 0.0 ? maxabs <= d.mtol : rel <= d.tol;
+    *record = true;
+    if (!d.fixed && finite && met && d.confirm) {
+        d.pending = 1;                      // the true residual decides (k_loop_confirm)
+        *record = false;
+        return false;
+    }
+    d.rel = rel;
+    d.maxabs = maxabs;
+    if (!finite) d.status = kLoopNonFinite;
+    else if (!d.fixed && met) d.status = kLoopDone;
+    else if (d.m >= d.limit) d.status = d.fixed ? kLoopDone : kLoopNotConverged;
+    else return true;
+    return false;
+}
 
 // ---- fused super-step, FP32 (kernels_fused.cu) -----------------------------
 constexpr int kFusedMaxS = 6;
@@ -216,29 +239,64 @@ cudaError_t launch_coarse_solve(const CoarseParams& p, cudaStream_t st);
 // Raise the dynamic shared-memory limit of the coarse kernels (once per process).
 cudaError_t coarse_configure();
 
-// ---- the two coarsest levels in one cluster launch (kernels_cluster.cu) ------
-constexpr int kBottomMaxS = 32;          // smoothing stages the coefficient table holds
-struct BottomParams {
-    int nx, ny, nz;                      // level B; level C = B + 1 has half of each
-    int per[3];                          // periodic flag per axis
-    float hx, hy, hz;                    // 1 / h^2 of level B
-    float chx, chy, chz;                 // 1 / h^2 of level C
-    int order, s, n_pre, n_post;         // smoothing of level B
-    float tau, mut1;                     // first stage: z = tau (L Y0 - f), Y1 = Y0 + mut1 z
-    float mu[kBottomMaxS + 1], nu[kBottomMaxS + 1], mut_tau[kBottomMaxS + 1];
-    float c0[kBottomMaxS + 1], gt[kBottomMaxS + 1];
-    int remove_mean;                     // every axis periodic: f_C -= mean(f_C)
+// ---- the coarse end of the V-cycle in one cluster launch (kernels_cluster.cu) --
+constexpr int kTailMaxS = 32;            // smoothing stages the coefficient table holds
+constexpr int kTailMaxLevels = 12;
+constexpr long long kTailWhole = 2560;   // cells of a level that every CTA holds whole (four a thread)
+constexpr long long kTailWhole64 = 64;   // the same in FP64: its arithmetic is worth splitting over more SMs
+constexpr long long kTailCells64 = 16384;    // FP64: cells up to which 16 SMs beat a launch per stage on all of them
+template <typename T>
+constexpr int tail_threads() {           // largest block, by the registers of a thread's cells
+    return sizeof(T) == 8 ? 512 : 640;
+}
+template <typename T>
+struct TailLevel {
+    int nx, ny, nz;                      // two-dimensional levels: nx x 1 x ny
+    int n_pre, n_post;
+    T hx, hy, hz, md;                    // 1 / h^2, -2 (hx + hy + hz)
+    T tau, omega, inv_cells;
+    int split;                           // cut into z slabs over the cluster
+    int group;                           // threads that work on it: 0 the whole CTA, 1 four warps, 2 one warp
+    int row, fld, buf, f;                // row stride, size of a buffer, offsets of the two buffers and of f
+    float inv_nq, inv_ny, inv_pairs;     // 1 / (nx / 2), 1 / ny (two-dimensional: 1), 1 / (nz / 2)
+    short first[17];                     // first plane pair of each CTA (split levels)
+};
+template <typename T>
+struct TailParams {
+    int nl;                              // levels, finest first
+    int per[3];
+    int order, s, gsrb;
+    T mut1, mu[kTailMaxS + 1], nu[kTailMaxS + 1], mut[kTailMaxS + 1], c0[kTailMaxS + 1], gt[kTailMaxS + 1];
+    int remove_mean;                     // every axis periodic: f -= mean(f) below the first level
     const int* sched;                    // coarse solve: s per super-step (device)
     int max_ss;
-    float tol;                           // relative residual stop, 0 = fixed count
-    float tau_unit;                      // coarse: mu~_j tau = mu_j * tau_unit
-    const float* rhs;                    // f_B (device)
-    float* u_out;                        // e_B (device)
+    T tol, tau_unit;                     // relative residual stop (0 = fixed count); mu~_j tau = mu_j tau_unit
+    const T* rhs;                        // f of the first level (device)
+    T* u_out;                            // its e (device)
     int* ss_done;                        // coarse super-steps done (device int)
+    TailLevel<T> lv[kTailMaxLevels];
+    // The whole inner loop of a mixed solve in this launch (FP32, the first level is
+    // level 0): the loop's state (nullptr: one V-cycle), phi and the carried FP64
+    // residual r = f - A phi of level 0, 1 / h^2 in FP64.
+    DeviceLoop* loop;
+    double* phi;
+    double* r64;
+    double ihx2, ihy2, ihz2;
+    int resident_off;                    // words to the copies of phi and r in shared memory
 };
-cudaError_t bottom_configure();
-// Cluster size (0: not possible), block size and shared memory for level B.
-int bottom_plan(int nx, int ny, int nz, int s, int* threads, size_t* bytes);
-cudaError_t launch_bottom(const BottomParams& p, int nc, int threads, size_t bytes, cudaStream_t st);
+struct TailLaunch {
+    int nc, threads;
+    size_t bytes;
+};
+cudaError_t tail_configure();
+// Bounded waits of this launch that gave up since the library was loaded; each wrote a NaN into its output.
+unsigned tail_wait_failures();
+// Fills the layout of p.lv (sizes and nl set) and the launch shape; false where
+// the levels (and, when p.loop is set, phi and r of the first one) do not fit one
+// cluster.
+template <typename T>
+bool tail_plan(TailParams<T>& p, bool twod, TailLaunch* t);
+template <typename T>
+cudaError_t launch_tail(const TailParams<T>& p, bool twod, const TailLaunch& t, cudaStream_t st);
 
 }  // namespace sg
