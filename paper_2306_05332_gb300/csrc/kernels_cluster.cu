@@ -547,7 +547,7 @@ __global__ void __launch_bounds__(tail_threads<T>()) k_tail_levels(const __grid_
             V nf[2], prev[2];
             nf[0] = nf[1] = c[0] = c[1] = prev[0] = prev[1] = mk2(T(0), T(0));
             if (h.act) load_nf(h, L, nf);
-            if (p.remove_mean) level_mean(h, L, nf);
+            if (nl > 1 && p.remove_mean) level_mean(h, L, nf);
             const T tu = p.tau_unit;
             auto sq = [&](const V (&l)[2]) {
                 return fmat(l[0].x, l[0].x, fmat(l[0].y, l[0].y, fmat(l[1].x, l[1].x, l[1].y * l[1].y)));
@@ -879,18 +879,22 @@ int row_stride(int nx, bool twod) {
 }  // namespace
 
 cudaError_t tail_configure() {
+    static bool configured = false;              // (the caller holds a lock)
+    if (configured) return cudaSuccess;
     cudaError_t e;
     if ((e = configure_one<float, false>()) != cudaSuccess) return e;
     if ((e = configure_one<float, true>()) != cudaSuccess) return e;
     if ((e = configure_one<double, false>()) != cudaSuccess) return e;
-    return configure_one<double, true>();
+    if ((e = configure_one<double, true>()) != cudaSuccess) return e;
+    configured = true;
+    return cudaSuccess;
 }
 
 // Layout of levels lv[0 .. nl) (nx, ny, nz set; two-dimensional ones as nx x 1 x ny)
 // in the shared memory of a cluster: false where they do not fit.
 template <typename T>
 bool tail_plan(TailParams<T>& p, bool twod, TailLaunch* out) {
-    if (p.nl < 2 || p.nl > kTailMaxLevels) return false;
+    if (p.nl < 1 || p.nl > kTailMaxLevels) return false;
     const int cap = tail_threads<T>();
     const unsigned sizes = twod ? TailCaps<T, true>::sizes : TailCaps<T, false>::sizes;
     const long long whole = sizeof(T) == 8 ? kTailWhole64 : kTailWhole;

@@ -30,7 +30,11 @@ template <> struct Acc<double> { using type = double; };
 __device__ __forceinline__ float acc_fma(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double acc_fma(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float acc_max(float a, float b) { return fmaxf(a, b); }
-__device__ __forceinline__ double acc_max(double a, double b) { return fmax(a, b); }
+// (of magnitudes: non-negative doubles compare as their bits, which keeps the
+// comparison off the FP64 pipe)
+__device__ __forceinline__ double acc_max(double a, double b) {
+    return __longlong_as_double(max(__double_as_longlong(a), __double_as_longlong(b)));
+}
 __device__ __forceinline__ float acc_abs(float a) { return fabsf(a); }
 __device__ __forceinline__ double acc_abs(double a) { return fabs(a); }
 
@@ -118,6 +122,12 @@ struct CoefT {
 };
 
 int kchunk_for(const LevelGeom& g, int bx, int by);
+
+bool has_faces(const LevelGeom& g) {
+    for (int f = 0; f < 6; ++f)
+        if (g.face[f]) return true;
+    return false;
+}
 
 // z-chunk with an even length (restriction and prolongation work on plane pairs).
 int even_kchunk(const LevelGeom& g) {
@@ -222,6 +232,183 @@ k_stage4(const LevelGeom g, const CoefT<float> cf, const float* __restrict__ ym1
         zm = c;
         c = zp;
     }
+}
+
+// ---------------------------------------------------------------------------
+// One RKL stage in FP64 (the stages of k_stage, every ghost rule).
+//
+// What bounds it.  GB300 issues two FP64 operations a clock and SM (0.63 T per second
+// on the chip): 16.7 M cells at one operation each are 27 us, the six arrays of a
+// later RKL2 stage (805 MB) 119 us.  So operations per cell decide.  The stage of
+// k_stage takes 16; here a stage takes 9 (first), 12 (second) or 13 with the same h
+// on every axis, 10, 13 or 14 otherwise:
+//   * the second difference of an axis as -2 c + (xm + xp), one addition and one FMA
+//     (two additions and a share of 2 c before); with equal h the axes' sums join
+//     before they are scaled (-4 c + (x + y sums), then z);
+//   * f, Z0 = L Y0 - f, Y0 and Y_{j-2} enter by one FMA each, with coefficients
+//     prepared on the host (Z0 is stored without the factor tau); in the second stage
+//     Y_{j-2} is Y0.
+// The terms are added from the small ones (differences, Z0, f) to the large ones
+// (Y0, Y_{j-2}, Y_{j-1}), so fewer roundings fall on values of the size of Y: against
+// 80-bit arithmetic one RKL2 super-step of s = 3 on a smooth field is off by 1.3e-16
+// relative (1.65e-16 with equal h), 1.76e-16 by k_stage's order.
+// 256^3, s = 3: the three stages took 468, 560 and 560 us by k_stage, 315, 413 and 447
+// us here, the FP64 pipe 83% busy.
+// V = 2: strips of two x cells (even nx, 16-byte aligned arrays).
+// ---------------------------------------------------------------------------
+struct Stage64 {
+    double m1t;             // first stage: Y1 = c + m1t Z0
+    double mu, ax, ay, az;  // later: mu c + mu~ tau / h^2 (second differences) ...
+    double kf, kz, k0, km;  // ... + kf f + kz Z0 + k0 Y0 + km Y_{j-2}
+};
+
+template <int V, int ORDER, bool FIRST, bool M2, bool FACES, bool UNIFORM>
+__global__ void __launch_bounds__(BX * BY)
+k_stage64(const LevelGeom g, const Stage64 cf, const double* __restrict__ ym1, const double* ym2, const double* y0,
+          const double* z0, const double* __restrict__ rhs, double* out, double* z0_out, int kchunk) {
+    const int i = (blockIdx.x * BX + threadIdx.x) * V;
+    const int j = blockIdx.y * BY + threadIdx.y;
+    const int nx = g.nx, ny = g.ny, nz = g.nz;
+    if (i >= nx || j >= ny) return;
+    const int k0 = blockIdx.z * kchunk, k1 = min(k0 + kchunk, nz);
+    const int plane = nx * ny;
+    int idx = k0 * plane + j * nx + i;
+    struct D {
+        double v[V];
+    };
+    auto ld = [](const double* p) {
+        D d;
+        if constexpr (V == 2) {
+            const double2 t = ld_d2(p);
+            d.v[0] = t.x;
+            d.v[1] = t.y;
+        } else {
+            d.v[0] = p[0];
+        }
+        return d;
+    };
+    auto st = [](double* p, const D& d) {
+        if constexpr (V == 2) *reinterpret_cast<double2*>(p) = make_double2(d.v[0], d.v[1]);
+        else p[0] = d.v[0];
+    };
+    // the strip beyond a wall: 2 face - c, or -c without face data
+    auto wall = [&](const double* face, const D& c) {
+        D d;
+#pragma unroll
+        for (int e = 0; e < V; ++e) d.v[e] = FACES && face ? fma(2.0, face[e], -c.v[e]) : -c.v[e];
+        return d;
+    };
+    const int yz = j * nx + i;                  // in a z face
+    D c = ld(ym1 + idx);
+    D zm = k0 > 0 ? ld(ym1 + idx - plane) : (g.per[2] ? ld(ym1 + idx + (nz - 1) * plane) : wall(FACES && g.face[4] ? g.face[4] + yz : nullptr, c));
+    for (int k = k0; k < k1; ++k, idx += plane) {
+        const D zp = k < nz - 1 ? ld(ym1 + idx + plane)
+                                : (g.per[2] ? ld(ym1 + idx - (nz - 1) * plane) : wall(FACES && g.face[5] ? g.face[5] + yz : nullptr, c));
+        const D ym = j > 0 ? ld(ym1 + idx - nx)
+                           : (g.per[1] ? ld(ym1 + idx + (ny - 1) * nx) : wall(FACES && g.face[2] ? g.face[2] + k * nx + i : nullptr, c));
+        const D yp = j < ny - 1 ? ld(ym1 + idx + nx)
+                                : (g.per[1] ? ld(ym1 + idx - (ny - 1) * nx) : wall(FACES && g.face[3] ? g.face[3] + k * nx + i : nullptr, c));
+        double xl, xr;
+        if (i > 0) xl = ym1[idx - 1];
+        else if (g.per[0]) xl = ym1[idx + nx - 1];
+        else xl = FACES && g.face[0] ? fma(2.0, g.face[0][k * ny + j], -c.v[0]) : -c.v[0];
+        if (i + V < nx) xr = ym1[idx + V];
+        else if (g.per[0]) xr = ym1[idx + V - nx];
+        else xr = FACES && g.face[1] ? fma(2.0, g.face[1][k * ny + j], -c.v[V - 1]) : -c.v[V - 1];
+        const D f = ld(rhs + idx);
+        D o, zo, a, b, m;
+        if (!FIRST && ORDER == 2) {
+            a = ld(y0 + idx);
+            b = ld(z0 + idx);
+        }
+        if (!FIRST && M2) m = ld(ym2 + idx);
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+            const double cc = c.v[e];
+            const double sx = (e > 0 ? c.v[e - 1] : xl) + (e + 1 < V ? c.v[e + 1 < V ? e + 1 : e] : xr);
+            const double sy = ym.v[e] + yp.v[e], sz = zm.v[e] + zp.v[e];
+            double t;
+            if (FIRST) t = -f.v[e];
+            else if (ORDER == 2) t = fma(cf.kz, b.v[e], cf.kf * f.v[e]);
+            else t = cf.kf * f.v[e];
+            if (UNIFORM) {
+                t = fma(cf.ax, fma(-4.0, cc, sx + sy) + fma(-2.0, cc, sz), t);
+            } else {
+                t = fma(cf.az, fma(-2.0, cc, sz), t);
+                t = fma(cf.ay, fma(-2.0, cc, sy), t);
+                t = fma(cf.ax, fma(-2.0, cc, sx), t);
+            }
+            if (FIRST) {
+                zo.v[e] = t;
+                o.v[e] = fma(cf.m1t, t, cc);
+            } else {
+                if (ORDER == 2) t = fma(cf.k0, a.v[e], t);
+                if (M2) t = fma(cf.km, m.v[e], t);
+                o.v[e] = fma(cf.mu, cc, t);
+            }
+        }
+        st(out + idx, o);
+        if (FIRST && ORDER == 2) st(z0_out + idx, zo);
+        zm = c;
+        c = zp;
+    }
+}
+
+template <int V, int ORDER, bool FIRST, bool M2>
+void launch_stage64_f(bool faces, bool uniform, dim3 grid, dim3 block, cudaStream_t st, const LevelGeom& g,
+                      const Stage64& cf, const double* ym1, const double* ym2, const double* y0, const double* z0,
+                      const double* rhs, double* out, double* z0_out, int kc) {
+    auto go = [&](auto f, auto u) {
+        k_stage64<V, ORDER, FIRST, M2, decltype(f)::value, decltype(u)::value>
+            <<<grid, block, 0, st>>>(g, cf, ym1, ym2, y0, z0, rhs, out, z0_out, kc);
+    };
+    if (faces) uniform ? go(std::true_type{}, std::true_type{}) : go(std::true_type{}, std::false_type{});
+    else uniform ? go(std::false_type{}, std::true_type{}) : go(std::false_type{}, std::false_type{});
+}
+
+template <int V>
+void launch_stage64_v(int order, bool first, bool faces, bool uniform, dim3 grid, dim3 block, cudaStream_t st,
+                      const LevelGeom& g, const Stage64& cf, const double* ym1, const double* ym2, const double* y0,
+                      const double* z0, const double* rhs, double* out, double* z0_out, int kc) {
+    auto go = [&](auto o, auto fi, auto m2) {
+        launch_stage64_f<V, decltype(o)::value, decltype(fi)::value, decltype(m2)::value>(
+            faces, uniform, grid, block, st, g, cf, ym1, ym2, y0, z0, rhs, out, z0_out, kc);
+    };
+    using One = std::integral_constant<int, 1>;
+    using Two = std::integral_constant<int, 2>;
+    if (first) order == 1 ? go(One{}, std::true_type{}, std::false_type{}) : go(Two{}, std::true_type{}, std::false_type{});
+    else if (order == 1) go(One{}, std::false_type{}, std::true_type{});
+    else if (ym2 == y0) go(Two{}, std::false_type{}, std::false_type{});
+    else go(Two{}, std::false_type{}, std::true_type{});
+}
+
+// c.tau is 1 and c.mut1, c.gt carry the factor tau (superstep): Z0 = L Y0 - f.
+cudaError_t launch_stage64(const LevelGeom& g, int order, bool first, const StageCoef& c, const double* ym1,
+                           const double* ym2, const double* y0, const double* z0, const double* rhs, double* out,
+                           double* z0_out, cudaStream_t st) {
+    Stage64 cf{};
+    cf.m1t = c.mut1;
+    cf.mu = c.mu;
+    const double w = first ? 1.0 : c.mut_tau;
+    cf.ax = w * g.ihx2;
+    cf.ay = w * g.ihy2;
+    cf.az = w * g.ihz2;
+    cf.kf = -c.mut_tau;
+    cf.kz = c.gt;
+    cf.k0 = c.c0;
+    cf.km = c.nu;
+    if (order == 2 && !first && ym2 == y0) cf.k0 = c.c0 + c.nu;
+    const bool faces = has_faces(g), uniform = g.ihx2 == g.ihy2 && g.ihy2 == g.ihz2;
+    const uintptr_t al = reinterpret_cast<uintptr_t>(ym1) | reinterpret_cast<uintptr_t>(ym2) |
+                         reinterpret_cast<uintptr_t>(y0) | reinterpret_cast<uintptr_t>(z0) |
+                         reinterpret_cast<uintptr_t>(rhs) | reinterpret_cast<uintptr_t>(out) |
+                         reinterpret_cast<uintptr_t>(z0_out);
+    const bool two = (g.nx & 1) == 0 && (al & 15) == 0;
+    const int bx = two ? 2 * BX : BX, kc = kchunk_for(g, bx, BY);
+    const dim3 block(BX, BY, 1), grid((g.nx + bx - 1) / bx, (g.ny + BY - 1) / BY, (g.nz + kc - 1) / kc);
+    if (two) launch_stage64_v<2>(order, first, faces, uniform, grid, block, st, g, cf, ym1, ym2, y0, z0, rhs, out, z0_out, kc);
+    else launch_stage64_v<1>(order, first, faces, uniform, grid, block, st, g, cf, ym1, ym2, y0, z0, rhs, out, z0_out, kc);
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -767,7 +954,7 @@ k_residual_zero(const LevelGeom g, const double* __restrict__ rhs, TO* r_out, do
 // warps), and the coarse value (1/8 of it) is written once.  Needs even
 // nx, ny, nz (true on every level that has a coarser one).
 // ---------------------------------------------------------------------------
-template <typename T, bool FACES>
+template <typename T, bool FACES, int WANT>
 __global__ void __launch_bounds__(BX * BY)
 k_residual_restrict(const LevelGeom g, const T* __restrict__ u, const T* __restrict__ rhs, T* coarse,
                     Partial* partials, int kchunk) {
@@ -795,10 +982,14 @@ k_residual_restrict(const LevelGeom g, const T* __restrict__ u, const T* __restr
             const T zp = (k < g.nz - 1) ? u[idx + plane] : z_high<FACES>(u, g, i, j, idx, plane, c);
             T xm, xp, ym, yp;
             xy_neighbours<FACES>(u, g, i, j, k, idx, c, xm, xp, ym, yp);
-            r = rhs[idx] - lap7(c, xm, xp, ym, yp, zm, zp, ihx2, ihy2, ihz2);
-            const A ra = A(r);
-            sq += ra * ra;
-            mx = acc_max(mx, acc_abs(ra));
+            // f - L u with the differences of lap7 (f enters by the FMAs)
+            const T two_c = T(2) * c;
+            r = acc_fma(-ihx2, (xm - two_c) + xp, acc_fma(-ihy2, (ym - two_c) + yp, acc_fma(-ihz2, (zm - two_c) + zp, rhs[idx])));
+            if (WANT == kWantNorms) {
+                const A ra = A(r);
+                sq += ra * ra;
+                mx = acc_max(mx, acc_abs(ra));
+            }
             zm = c;
             c = zp;
         }
@@ -813,13 +1004,13 @@ k_residual_restrict(const LevelGeom g, const T* __restrict__ u, const T* __restr
                 const T cval = (s_acc[threadIdx.y][threadIdx.x] + s_acc[threadIdx.y + 1][threadIdx.x]) * T(0.125);
                 const int I = i >> 1, J = j >> 1, K = k >> 1;
                 if (coarse) coarse[(K * cny + J) * cnx + I] = cval;
-                csum += A(cval);
+                if (WANT != kWantNothing) csum += A(cval);
             }
             __syncthreads();
         }
     }
     const int bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-    block_reduce_write<A>(sq, mx, csum, partials, bid);
+    if (WANT != kWantNothing) block_reduce_write<A>(sq, mx, csum, partials, bid);
 }
 
 // FP32 residual + restriction on homogeneous ghosts, for nx % 4 == 0 and
@@ -827,6 +1018,7 @@ k_residual_restrict(const LevelGeom g, const T* __restrict__ u, const T* __restr
 // rows (2J, 2J + 1) and streams z, so each 2 x 2 x 2 block of the 8-cell mean
 // (Eq. restriction_example_3D) is summed in its registers, with no shared
 // memory or barrier; the z neighbours are carried in registers.
+template <int WANT>
 __global__ void __launch_bounds__(BX * BY, 4)
 k_residual_restrict4(const LevelGeom g, const float* __restrict__ u, const float* __restrict__ rhs,
                      float* __restrict__ coarse, Partial* partials, int kchunk) {
@@ -866,17 +1058,19 @@ k_residual_restrict4(const LevelGeom g, const float* __restrict__ u, const float
             const float r5 = fb.y - lap7(cb.y, cb.x, cb.z, ca.y, yp.y, zb.y, zpb.y, hx, hy, hz);
             const float r6 = fb.z - lap7(cb.z, cb.y, cb.w, ca.z, yp.z, zb.z, zpb.z, hx, hy, hz);
             const float r7 = fb.w - lap7(cb.w, cb.z, xrb, ca.w, yp.w, zb.w, zpb.w, hx, hy, hz);
-            sq = fmaf(r0, r0, fmaf(r1, r1, fmaf(r2, r2, fmaf(r3, r3, sq))));
-            sq = fmaf(r4, r4, fmaf(r5, r5, fmaf(r6, r6, fmaf(r7, r7, sq))));
-            mx = fmaxf(mx, fmaxf(fmaxf(fmaxf(fabsf(r0), fabsf(r1)), fmaxf(fabsf(r2), fabsf(r3))),
-                                 fmaxf(fmaxf(fabsf(r4), fabsf(r5)), fmaxf(fabsf(r6), fabsf(r7)))));
+            if (WANT == kWantNorms) {
+                sq = fmaf(r0, r0, fmaf(r1, r1, fmaf(r2, r2, fmaf(r3, r3, sq))));
+                sq = fmaf(r4, r4, fmaf(r5, r5, fmaf(r6, r6, fmaf(r7, r7, sq))));
+                mx = fmaxf(mx, fmaxf(fmaxf(fmaxf(fabsf(r0), fabsf(r1)), fmaxf(fabsf(r2), fabsf(r3))),
+                                     fmaxf(fmaxf(fabsf(r4), fabsf(r5)), fmaxf(fabsf(r6), fabsf(r7)))));
+            }
             const float2 s2 = make_float2((r0 + r1) + (r4 + r5), (r2 + r3) + (r6 + r7));
             if ((k & 1) == 0) {
                 acc = s2;
             } else {
                 const float2 cv = make_float2((acc.x + s2.x) * 0.125f, (acc.y + s2.y) * 0.125f);
                 if (coarse) *reinterpret_cast<float2*>(coarse + ((k >> 1) * cny + jp) * cnx + 2 * q) = cv;
-                csum += cv.x + cv.y;
+                if (WANT != kWantNothing) csum += cv.x + cv.y;
             }
             za = ca;
             ca = zpa;
@@ -885,7 +1079,7 @@ k_residual_restrict4(const LevelGeom g, const float* __restrict__ u, const float
         }
     }
     const int bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-    block_reduce_write<float>(sq, mx, csum, partials, bid);
+    if (WANT != kWantNothing) block_reduce_write<float>(sq, mx, csum, partials, bid);
 }
 
 // ---------------------------------------------------------------------------
@@ -1869,12 +2063,6 @@ long long restrict_blocks(const LevelGeom& g) {
     return (long long)((g.nx + BX - 1) / BX) * ((g.ny + BY - 1) / BY) * ((g.nz + kc - 1) / kc);
 }
 
-bool has_faces(const LevelGeom& g) {
-    for (int f = 0; f < 6; ++f)
-        if (g.face[f]) return true;
-    return false;
-}
-
 template <typename T, int ORDER, bool FIRST>
 void launch_stage_f(bool faces, dim3 grid, dim3 block, cudaStream_t st, const LevelGeom& g, const CoefT<T>& cf,
                     const T* ym1, const T* ym2, const T* y0, const T* z0, const T* rhs, T* out, T* z0_out, int kc) {
@@ -1886,6 +2074,9 @@ template <typename T>
 cudaError_t launch_stage(const LevelGeom& g, int order, bool first, const StageCoef& c,
                          const T* ym1, const T* ym2, const T* y0, const T* z0, const T* rhs,
                          T* out, T* z0_out, cudaStream_t st) {
+    if constexpr (std::is_same<T, double>::value) {
+        return launch_stage64(g, order, first, c, ym1, ym2, y0, z0, rhs, out, z0_out, st);
+    } else {
     CoefT<T> cf;
     cf.tau = T(c.tau); cf.mut1 = T(c.mut1); cf.mu = T(c.mu); cf.nu = T(c.nu);
     cf.mut_tau = T(c.mut_tau); cf.c0 = T(c.c0); cf.gt = T(c.gt);
@@ -1922,6 +2113,7 @@ cudaError_t launch_stage(const LevelGeom& g, int order, bool first, const StageC
         else launch_stage_f<T, 2, false>(faces, grid, block, st, g, cf, ym1, ym2, y0, z0, rhs, out, z0_out, kc);
     }
     return cudaGetLastError();
+    }
 }
 
 template <typename TO>
@@ -1981,7 +2173,7 @@ cudaError_t launch_residual(const LevelGeom& g, const TI* u, const TI* rhs, TO* 
 
 template <typename T>
 cudaError_t launch_residual_restrict(const LevelGeom& g, const T* u, const T* rhs, T* coarse_out,
-                                     Partial* partials, int* nblocks_out, cudaStream_t st) {
+                                     Partial* partials, int* nblocks_out, cudaStream_t st, int want) {
     if (g.twod) {
         dim3 block(BX, BY, 1);
         dim3 grid((g.nx + BX - 1) / BX, (g.ny + BY - 1) / BY, 1);
@@ -2004,7 +2196,9 @@ cudaError_t launch_residual_restrict(const LevelGeom& g, const T* u, const T* rh
             while (kc < 16 && gx * gy * ((g.nz + 2 * kc - 1) / (2 * kc)) >= 3LL * sm_count()) kc *= 2;
             dim3 block(BX, BY, 1);
             dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)((g.nz + kc - 1) / kc));
-            k_residual_restrict4<<<grid, block, 0, st>>>(g, u, rhs, coarse_out, partials, kc);
+            if (want == kWantNorms) k_residual_restrict4<kWantNorms><<<grid, block, 0, st>>>(g, u, rhs, coarse_out, partials, kc);
+            else if (want == kWantSum) k_residual_restrict4<kWantSum><<<grid, block, 0, st>>>(g, u, rhs, coarse_out, partials, kc);
+            else k_residual_restrict4<kWantNothing><<<grid, block, 0, st>>>(g, u, rhs, coarse_out, partials, kc);
             if (nblocks_out) *nblocks_out = (int)(grid.x * grid.y * grid.z);
             return cudaGetLastError();
         }
@@ -2012,8 +2206,14 @@ cudaError_t launch_residual_restrict(const LevelGeom& g, const T* u, const T* rh
     const int kc = even_kchunk(g);
     dim3 block(BX, BY, 1);
     dim3 grid((g.nx + BX - 1) / BX, (g.ny + BY - 1) / BY, (g.nz + kc - 1) / kc);
-    if (has_faces(g)) k_residual_restrict<T, true><<<grid, block, 0, st>>>(g, u, rhs, coarse_out, partials, kc);
-    else k_residual_restrict<T, false><<<grid, block, 0, st>>>(g, u, rhs, coarse_out, partials, kc);
+    auto run = [&](auto faces) {
+        constexpr bool F = decltype(faces)::value;
+        if (want == kWantNorms) k_residual_restrict<T, F, kWantNorms><<<grid, block, 0, st>>>(g, u, rhs, coarse_out, partials, kc);
+        else if (want == kWantSum) k_residual_restrict<T, F, kWantSum><<<grid, block, 0, st>>>(g, u, rhs, coarse_out, partials, kc);
+        else k_residual_restrict<T, F, kWantNothing><<<grid, block, 0, st>>>(g, u, rhs, coarse_out, partials, kc);
+    };
+    if (has_faces(g)) run(std::true_type{});
+    else run(std::false_type{});
     if (nblocks_out) *nblocks_out = (int)(grid.x * grid.y * grid.z);
     return cudaGetLastError();
 }
@@ -2225,10 +2425,10 @@ template cudaError_t launch_residual<double, float>(const LevelGeom&, const doub
                                                     float*, Partial*, int*, cudaStream_t, double*);
 template cudaError_t launch_residual<float, float>(const LevelGeom&, const float*, const float*,
                                                    float*, Partial*, int*, cudaStream_t, float*);
-template cudaError_t launch_residual_restrict<float>(const LevelGeom&, const float*, const float*,
-                                                     float*, Partial*, int*, cudaStream_t);
-template cudaError_t launch_residual_restrict<double>(const LevelGeom&, const double*, const double*,
-                                                      double*, Partial*, int*, cudaStream_t);
+template cudaError_t launch_residual_restrict<float>(const LevelGeom&, const float*, const float*, float*, Partial*, int*,
+                                                      cudaStream_t, int);
+template cudaError_t launch_residual_restrict<double>(const LevelGeom&, const double*, const double*, double*, Partial*, int*,
+                                                      cudaStream_t, int);
 template cudaError_t launch_prolong_correct<float>(const LevelGeom&, const float*, float*, cudaStream_t);
 template cudaError_t launch_prolong_correct<double>(const LevelGeom&, const double*, double*,
                                                     cudaStream_t);

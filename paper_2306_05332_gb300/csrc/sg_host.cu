@@ -454,9 +454,11 @@ sg_status superstep(sg_grid* g, int l, int order, int s, double tau_frac, bool f
     const double tau = tau_frac * dtpar * r.tau_over_dtpar;
     W* t[3] = {(W*)L.t[0], (W*)L.t[1], (W*)L.t[2]};
     W* z0 = (W*)L.z0;
+    // FP64 stages keep Z0 = L Y0 - f without the factor tau (kernels_stencil.cu)
+    const bool bare = std::is_same<W, double>::value;
     StageCoef c{};
-    c.tau = tau;
-    c.mut1 = r.mut[1];
+    c.tau = bare ? 1.0 : tau;
+    c.mut1 = bare ? r.mut[1] * tau : r.mut[1];
     W* out1 = t[0];
     const int cls = l == 0 ? K_STAGE0 : K_STAGE_C;
     const double nb = double(L.n) * sizeof(W);
@@ -476,7 +478,7 @@ sg_status superstep(sg_grid* g, int l, int order, int s, double tau_frac, bool f
         cj.nu = r.nu[j];
         cj.mut_tau = r.mut[j] * tau;
         cj.c0 = r.c0[j];
-        cj.gt = r.gt[j];
+        cj.gt = bare ? r.gt[j] * tau : r.gt[j];
         const W* ym1 = (j - 1 == 0) ? u : t[(j - 2) % 3];
         const W* ym2 = (j - 2 == 0) ? u : t[(j - 3) % 3];
         W* out = (j == s) ? u : t[(j - 1) % 3];
@@ -706,7 +708,9 @@ int tail_level(const sg_grid* g, int L, TailParams<W>& p, TailLaunch* t) {
             g->lv[L - 1].nx % 4 != 0 || (long long)g->lv[b].nx * g->lv[b].ny > 1024)
             return -1;
     }
-    for (; b <= L - 2; ++b)
+    // FP64: also the coarsest level alone (16^3: 0.70 ms a solve on one SM, whose FP64
+    // rate bounds it)
+    for (; b <= (std::is_same<W, float>::value ? L - 2 : L - 1); ++b)
         if (tail_params<W>(g, L, b, p, t)) return b;
     return -1;
 }
@@ -790,7 +794,8 @@ sg_status vcycle(sg_grid* g, int L, W* u0, const W* rhs0, bool faces, bool zero0
         {
             ProfScope ps(g, K_RESTRICT, (2.0 + 0.125) * g->lv[l - 1].n * sizeof(W));
             SG_CK(launch_residual_restrict<W>(geom(g, l - 1, faces && l - 1 == 0), cur[l - 1], R(l - 1),
-                                              (W*)g->lv[l].rhs, g->partials, &nb, g->st));   // 2a, 2b
+                                              (W*)g->lv[l].rhs, g->partials, &nb, g->st,
+                                              per ? kWantSum : kWantNothing));               // 2a, 2b
         }
         ++g->launches;
         if (per) {                                                              // coarse mean removed

@@ -93,11 +93,15 @@ cudaError_t launch_residual_zero(const LevelGeom& g, const double* rhs, TO* r_ou
                                  int* nblocks_out, cudaStream_t st, double* r_full = nullptr,
                                  int* nkernels = nullptr);
 
-// Fused residual + 8-cell restriction (+ norm partials, + coarse sum partials).
+// Fused residual + 8-cell restriction.  `want`: the block partials it writes besides
+// (the norms of r and the sum of the coarse values; the sum alone; nothing: a
+// V-cycle reads the sum only where every axis is periodic, and the norms cost an FP64
+// level two operations a cell).
+constexpr int kWantNothing = 0, kWantSum = 1, kWantNorms = 2;
 template <typename T>
 cudaError_t launch_residual_restrict(const LevelGeom& fine, const T* u, const T* rhs,
                                      T* coarse_out, Partial* partials, int* nblocks_out,
-                                     cudaStream_t st);
+                                     cudaStream_t st, int want = kWantNorms);
 
 // fine += P(coarse) with coarse ghosts by the homogeneous/periodic rule.
 template <typename T>
