@@ -127,9 +127,10 @@ typedef struct sg_options {
     double max_residual_tol;/* > 0: stop when max |L phi - f| <= this (App. B's
                                test) instead of the relative L2 test; tol is then
                                ignored                                          [0]  */
-    int    tile_rows;       /* rows of the tile of the fused s = 2, 3 super-step:
-                               14 or 16; 0 = the launcher's cost model (the plan
-                               whose busiest SM has the least work)           [0]  */
+    int    tile_rows;       /* rows of the tile of the fused s = 2, 3 super-step
+                               with one stage per thread: 14 or 16; 0 = the kernel
+                               with one column per thread, tiles by its launcher's
+                               cost model (faster; the same bits)             [0]  */
     int    inner_n_pre;     /* smoothing super-steps on the way down on levels
                                1 .. L-2; -1 = n_pre (the paper's N_pre on every
                                level)                                           [-1] */
@@ -321,8 +322,7 @@ typedef struct sg_tune_entry {
  * every candidate (RKL order 1 and 2 -- or only the current order when
  * keep_order is 1 --, s = 2..6, a few tau fractions, fused on and off, and
  * (N_pre, N_post) = (2, 1), (3, 2), (4, 3) or (5, 3), on levels 1 .. L-2 the
- * same or (2, 1), and for the fused s = 2, 3 super-step both tile shapes,
- * 32 x 14 and 32 x 16) run
+ * same or (2, 1)) run
  * two and six V-cycles at `levels` (0 = the level rule), take the difference
  * of their CUDA-event times (so per-solve set-up drops out) and score the time
  * per decade of residual reduction over cycles 2..6, bounded below by the

@@ -400,7 +400,8 @@ cudaError_t fused_configure() {
     int dev = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = lean_configure()) != cudaSuccess) return e;       // s = 2, 3 (kernels_superstep.cu)
+    if ((e = columns_configure()) != cudaSuccess) return e;    // s = 2, 3 (kernels_columns.cu)
+    if ((e = lean_configure()) != cudaSuccess) return e;       // s = 2, 3 on request (kernels_superstep.cu)
     if ((e = configure_s<4>()) != cudaSuccess) return e;
     if ((e = configure_s<5>()) != cudaSuccess) return e;
     return configure_s<6>();
@@ -411,7 +412,9 @@ cudaError_t launch_superstep_fused(const LevelGeom& g, int order, int s, bool ze
                                    bool tma) {
     switch (s) {
         case 2:
-        case 3: return launch_superstep_lean(g, order, s, zero_y0, cf, y0, f, out, st, tile_rows, tma);
+        case 3:
+            if (tile_rows == 0 && !tma) return launch_superstep_columns(g, order, s, zero_y0, cf, y0, f, out, st);
+            return launch_superstep_lean(g, order, s, zero_y0, cf, y0, f, out, st, tile_rows, tma);
         case 4: return dispatch<4>(order, zero_y0, g, cf, y0, f, out, st);
         case 5: return dispatch<5>(order, zero_y0, g, cf, y0, f, out, st);
         case 6: return dispatch<6>(order, zero_y0, g, cf, y0, f, out, st);

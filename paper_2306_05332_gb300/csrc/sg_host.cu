@@ -592,9 +592,10 @@ sg_status coarse_solve(sg_grid* g, int l, const W* rhs, W* u, int* d_done) {
 }
 
 // One fused super-step (FP32, homogeneous or periodic ghosts): out = Y_s(y0),
-// y0 == nullptr meaning Y0 = 0.
+// y0 == nullptr meaning Y0 = 0.  by_options: the kernel that tile_rows and staging ask
+// for, otherwise the one with a column per thread (the same bits).
 sg_status superstep_fused(sg_grid* g, int l, int order, int s, double tau_frac, const float* y0,
-                          const float* rhs, float* out) {
+                          const float* rhs, float* out, bool by_options) {
     const Level& L = g->lv[l];
     const Rkl r = make_rkl(order, s);
     const double tau = tau_frac * (2.0 / lambda_max(L)) * r.tau_over_dtpar;
@@ -611,24 +612,28 @@ sg_status superstep_fused(sg_grid* g, int l, int order, int s, double tau_frac, 
     {
         ProfScope ps(g, l == 0 ? K_STAGE0 : K_STAGE_C, double(L.n) * sizeof(float) * (y0 ? 3 : 2));
         SG_CK(launch_superstep_fused(geom(g, l, false), order, s, y0 == nullptr, cf, y0, rhs, out, g->st,
-                                     g->opt.tile_rows, g->opt.staging == SG_STAGE_TMA));
+                                     by_options ? g->opt.tile_rows : 0,
+                                     by_options && g->opt.staging == SG_STAGE_TMA));
     }
     ++g->launches;
     return SG_OK;
 }
 
-// The fused super-step streams each tile through all s stages one plane at a
-// time; on small levels that serial chain of planes (its pipeline fill on
-// short z chunks) costs more than it saves in HBM traffic (the level is
-// L2-resident anyway), so only levels with at least kFusedMinCells cells use
-// it: with the strip stage kernel, 128^3 runs faster as one launch per stage
-// (7.72 against 7.85 ms per 256^3 solve).
+// A fused super-step streams each tile through all s stages one plane at a time; on
+// small levels that serial chain of planes (and the pipeline's fill on short z chunks)
+// costs more than the launches and the L2 traffic it saves.  s = 3, one column per
+// thread: 128^3 16.5 us against 3 launches of 7 - 8 us, 96^3 12.4 against about 12, 64^3
+// 8.3 against 8; solves with the line at 2^22, 2^21, 2^19 and 2^17 cells: 128^3 3102, 2895,
+// 2884 and 2856 us, 112 x 80 x 144 2264, 2264, 2204 and 2180, 64 uneven grids at once
+// 54.1, 49.5, 47.2 and 48.1 ms.  s = 2 (128^3 14.4 us against 2 launches of 6) and the
+// kernel for s = 4 .. 6 only gain on large levels.
 constexpr long long kFusedMinCells = 1LL << 22;
+constexpr long long kColumnMinCells = 1LL << 17;
 
 bool use_fused(const sg_grid* g, bool faces, int l) {
     return !g->twod && g->precision == SG_MIXED && g->opt.fused && !faces && g->opt.smoother == SG_SMOOTH_RKL &&
            fused_supported(g->opt.rkl_order, g->opt.s_smooth) &&
-           g->lv[l].n >= kFusedMinCells;
+           g->lv[l].n >= (g->opt.s_smooth == 3 ? kColumnMinCells : kFusedMinCells);
 }
 
 // The first super-step of a level's pre-smoothing starts from Y0 = 0: for
@@ -766,7 +771,7 @@ sg_status vcycle(sg_grid* g, int L, W* u0, const W* rhs0, bool faces, bool zero0
                     const bool z = zero_start && c == 0;
                     float* out = z ? cur[l] : alt[l];
                     SG_TRY(superstep_fused(g, l, g->opt.rkl_order, g->opt.s_smooth, g->opt.tau_frac,
-                                           z ? nullptr : cur[l], R(l), out));
+                                           z ? nullptr : cur[l], R(l), out, g->lv[l].n >= kFusedMinCells));
                     if (!z) std::swap(cur[l], alt[l]);
                 }
                 if (zero_start && count == 0) SG_CK(cudaMemsetAsync(cur[l], 0, g->lv[l].n * sizeof(W), g->st));
@@ -774,7 +779,7 @@ sg_status vcycle(sg_grid* g, int L, W* u0, const W* rhs0, bool faces, bool zero0
             }
             if (zero_start && count > 0 && use_fused_zero(g, fc, l)) {
                 SG_TRY(superstep_fused(g, l, g->opt.rkl_order, g->opt.s_smooth, g->opt.tau_frac, nullptr, R(l),
-                                       cur[l]));
+                                       cur[l], false));
                 return relax<W>(g, l, count - 1, fc, cur[l], R(l));
             }
         }
@@ -1967,12 +1972,7 @@ sg_status sg_autotune(sg_grid* g, int levels, int keep_order, sg_tune_entry* tab
                         for (int in = 0; in < 2; ++in) {      // inner levels: the same counts, or (2, 1)
                             const int ip = in ? 2 : -1, iq = in ? 1 : -1;
                             if (in && pc[0] == 2 && pc[1] == 1) continue;
-                            if (fz && s <= 3 && !g->twod) {      // the tile shapes of the fused s = 2, 3 kernel
-                                cands.push_back({order, s, fz, cs[ic], pc[0], pc[1], 14, ip, iq});
-                                cands.push_back({order, s, fz, cs[ic], pc[0], pc[1], 16, ip, iq});
-                            } else {
-                                cands.push_back({order, s, fz, cs[ic], pc[0], pc[1], 0, ip, iq});
-                            }
+                            cands.push_back({order, s, fz, cs[ic], pc[0], pc[1], 0, ip, iq});
                         }
         }
     }
@@ -2078,7 +2078,7 @@ sg_status sg_op_superstep(sg_grid* g, int level, int dtype, int order, int s, do
         return fail(SG_ERR_ARG, "bad order / s / tau_frac");
     const bool faces = !homogeneous && level == 0 && g->have_faces;
     if (dtype == 1 && g->opt.fused && !faces && !g->twod && fused_supported(order, s))
-        return superstep_fused(g, level, order, s, tau_frac, (const float*)u, (const float*)rhs, (float*)out);
+        return superstep_fused(g, level, order, s, tau_frac, (const float*)u, (const float*)rhs, (float*)out, true);
     if (!u) return fail(SG_ERR_ARG, "u == NULL (zero initial guess) needs the fused FP32 super-step");
     const size_t bytes = g->lv[level].n * (dtype == 0 ? 8 : 4);
     SG_CK(cudaMemcpyAsync(out, u, bytes, cudaMemcpyDeviceToDevice, g->st));

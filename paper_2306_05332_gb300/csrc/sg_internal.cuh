@@ -218,6 +218,10 @@ cudaError_t lean_configure();
 cudaError_t launch_superstep_lean(const LevelGeom& g, int order, int s, bool zero_y0, const FusedCoef& cf,
                                   const float* y0, const float* f, float* out, cudaStream_t st, int tile_rows,
                                   bool tma);
+// s = 2, 3: one thread per column (kernels_columns.cu).
+cudaError_t columns_configure();
+cudaError_t launch_superstep_columns(const LevelGeom& g, int order, int s, bool zero_y0, const FusedCoef& cf,
+                                     const float* y0, const float* f, float* out, cudaStream_t st);
 // Launches of the TMA path that gave up a bounded wait (or found their shared
 // memory misaligned) since the library was loaded; each wrote a NaN into its
 // output, so the solve that ran it reports a non-finite residual.
