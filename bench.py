@@ -246,8 +246,8 @@ def hbm_peak():
 
 
 # Source files of the kernel whose DRAM bytes `roofline.traffic` reports (the
-# fused level-0 super-step) and the header it includes.
-TRAFFIC_SOURCES = ("kernels_superstep.cu", "sg_internal.cuh")
+# fused level-0 super-step) and the headers it includes.
+TRAFFIC_SOURCES = ("kernels_columns.cu", "sg_superstep.cuh", "sg_internal.cuh")
 
 
 def kernel_source_hash():

@@ -1,6 +1,6 @@
 // The outer convergence loop of Sec. 2.1 on the device: V-cycles repeat while
 // the relative residual ||L phi - f|| / ||L 0 - f|| is above the tolerance
-// (Sec. 4.1), decided by one-thread kernels that set the conditions of the
+// (Sec. 4.1), decided by one-block kernels that set the conditions of the
 // WHILE nodes of a CUDA graph, so a solve (or a batch of them) runs without a
 // host round trip per cycle.  The decisions are those of the host loop:
 //   * after each cycle: the relative residual (mixed precision: of the FP64
@@ -9,6 +9,7 @@
 //     inner loop so that the true FP64 residual is computed once and
 //     confirmed (or the cycles resume from it);
 //   * a non-finite residual, the cycle cap or a fixed cycle count end it.
+#include "sg_fold.cuh"
 #include "sg_internal.cuh"
 
 namespace sg {
@@ -29,9 +30,13 @@ __device__ __forceinline__ void loop_record(DeviceLoop& d, double rel, double ma
     d.maxabs = maxabs;
 }
 
-// After a cycle: count it and decide whether the inner loop runs another.
-__global__ void k_loop_step(DeviceLoop* dl, const Reduced* red, const int* ss_done, const int* sched,
-                            cudaGraphConditionalHandle inner) {
+// After a cycle: fold the residual's block partials (a launch of its own cost 2.5 us a
+// cycle), count the cycle and decide whether the inner loop runs another.
+__global__ void __launch_bounds__(kRedThreads)
+k_loop_step(DeviceLoop* dl, const Partial* partials, int nb, Reduced* red, const int* ss_done, const int* sched,
+            cudaGraphConditionalHandle inner) {
+    fold_partials(partials, nb, red);
+    if (threadIdx.x != 0) return;
     DeviceLoop& d = *dl;
     const int ss = ss_done ? *ss_done : 0;
     if (d.m < kLoopHistory) d.coarse_ss[d.m] = ss;
@@ -46,8 +51,12 @@ __global__ void k_loop_step(DeviceLoop* dl, const Reduced* red, const int* ss_do
 
 // After the inner loop (mixed precision: the true FP64 residual is in red):
 // confirm, or resume the cycles.
-__global__ void k_loop_confirm(DeviceLoop* dl, const Reduced* red, cudaGraphConditionalHandle outer,
-                               cudaGraphConditionalHandle inner, int has_inner) {
+// (nb > 0: the residual's partials)
+__global__ void __launch_bounds__(kRedThreads)
+k_loop_confirm(DeviceLoop* dl, const Partial* partials, int nb, Reduced* red, cudaGraphConditionalHandle outer,
+               cudaGraphConditionalHandle inner, int has_inner) {
+    if (nb > 0) fold_partials(partials, nb, red);
+    if (threadIdx.x != 0) return;
     DeviceLoop& d = *dl;
     unsigned go = 0;
     d.confirms += 1;
@@ -81,15 +90,16 @@ cudaError_t launch_loop_init(const DeviceLoop* d, cudaGraphConditionalHandle out
     return cudaGetLastError();
 }
 
-cudaError_t launch_loop_step(DeviceLoop* d, const Reduced* red, const int* ss_done, const int* sched,
-                             cudaGraphConditionalHandle inner, cudaStream_t st) {
-    k_loop_step<<<1, 1, 0, st>>>(d, red, ss_done, sched, inner);
+cudaError_t launch_loop_step(DeviceLoop* d, const Partial* partials, int nb, Reduced* red, const int* ss_done,
+                             const int* sched, cudaGraphConditionalHandle inner, cudaStream_t st) {
+    k_loop_step<<<1, kRedThreads, 0, st>>>(d, partials, nb, red, ss_done, sched, inner);
     return cudaGetLastError();
 }
 
-cudaError_t launch_loop_confirm(DeviceLoop* d, const Reduced* red, cudaGraphConditionalHandle outer,
-                                cudaGraphConditionalHandle inner, bool has_inner, cudaStream_t st) {
-    k_loop_confirm<<<1, 1, 0, st>>>(d, red, outer, inner, has_inner ? 1 : 0);
+cudaError_t launch_loop_confirm(DeviceLoop* d, const Partial* partials, int nb, Reduced* red,
+                                cudaGraphConditionalHandle outer, cudaGraphConditionalHandle inner, bool has_inner,
+                                cudaStream_t st) {
+    k_loop_confirm<<<1, nb > 0 ? kRedThreads : 1, 0, st>>>(d, partials, nb, red, outer, inner, has_inner ? 1 : 0);
     return cudaGetLastError();
 }
 

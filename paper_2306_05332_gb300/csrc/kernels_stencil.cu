@@ -8,6 +8,7 @@
 // read from HBM once per sweep (x/y neighbours hit L1/L2), coalesced along x.
 // These are HBM-bandwidth-bound kernels; no tensor cores are involved.
 #include "sg_field_ops.cuh"
+#include "sg_fold.cuh"
 #include "sg_internal.cuh"
 #include "sg_update.cuh"
 
@@ -84,6 +85,33 @@ __device__ __forceinline__ T z_high(const T* u, const LevelGeom& g, int i, int j
 __device__ __forceinline__ float4 ld_f4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ double2 ld_d2(const double* p) { return *reinterpret_cast<const double2*>(p); }
 __device__ __forceinline__ float4 neg_f4(float4 v) { return make_float4(-v.x, -v.y, -v.z, -v.w); }
+
+// Strip q (of nq in a row) and row j of this thread.  Blocks of 32 x 8 strips leave lanes
+// idle where a row is no multiple of 32 strips (48: a quarter, 16: half); there the
+// plane's strips are numbered through and a block takes 256 consecutive ones (flat): the
+// GS-RB solve of 192^3 2430 -> 2329 us, 64 uneven grids 50.9 -> 46.7 ms.  Other rows keep
+// the 32 x 8 block, which re-reads fewer neighbour rows.
+__device__ __forceinline__ bool strip_at(int nq, int rows, int flat, int& q, int& j) {
+    if (flat) {
+        const int s = blockIdx.x * (BX * BY) + threadIdx.y * BX + threadIdx.x;
+        j = s / nq;
+        q = s - j * nq;
+    } else {
+        q = blockIdx.x * BX + threadIdx.x;
+        j = blockIdx.y * BY + threadIdx.y;
+    }
+    return q < nq && j < rows;
+}
+struct StripGrid {
+    int flat;
+    long long gx, gy;
+    StripGrid(int nq, int rows) : flat(nq % BX != 0), gx((nq + BX - 1) / BX), gy((rows + BY - 1) / BY) {
+        if (flat) {
+            gx = ((long long)nq * rows + BX * BY - 1) / (BX * BY);
+            gy = 1;
+        }
+    }
+};
 
 // Eq. discrete_laplace_3D from the six neighbours.
 template <typename T>
@@ -1021,12 +1049,11 @@ k_residual_restrict(const LevelGeom g, const T* __restrict__ u, const T* __restr
 template <int WANT>
 __global__ void __launch_bounds__(BX * BY, 4)
 k_residual_restrict4(const LevelGeom g, const float* __restrict__ u, const float* __restrict__ rhs,
-                     float* __restrict__ coarse, Partial* partials, int kchunk) {
-    const int q = blockIdx.x * BX + threadIdx.x;        // cells 4q .. 4q + 3
-    const int jp = blockIdx.y * BY + threadIdx.y;       // rows 2 jp, 2 jp + 1
+                     float* __restrict__ coarse, Partial* partials, int kchunk, int flat) {
+    int q, jp;                                          // cells 4q .. 4q + 3 of rows 2 jp, 2 jp + 1
     const int nx = g.nx, ny = g.ny, nz = g.nz;
     float sq = 0.0f, mx = 0.0f, csum = 0.0f;
-    if (4 * q < nx && 2 * jp < ny) {
+    if (strip_at(nx / 4, ny / 2, flat, q, jp)) {
         const int i0 = 4 * q, j0 = 2 * jp, plane = nx * ny;
         const int cnx = nx >> 1, cny = ny >> 1;
         const bool px = g.per[0] != 0, py = g.per[1] != 0, pz = g.per[2] != 0;
@@ -1214,11 +1241,11 @@ k_prolong_correct2d(const LevelGeom g, const T* __restrict__ coarse, T* fine_u) 
 // then the y interpolants of its two rows, and streams z with 16-byte
 // read-modify-writes of the fine strips.
 __global__ void __launch_bounds__(BX * BY)
-k_prolong_correct4(const LevelGeom g, const float* __restrict__ coarse, float* __restrict__ fine_u, int kchunk) {
-    const int q = blockIdx.x * BX + threadIdx.x;
-    const int J = blockIdx.y * BY + threadIdx.y;
+k_prolong_correct4(const LevelGeom g, const float* __restrict__ coarse, float* __restrict__ fine_u, int kchunk,
+                   int flat) {
+    int q, J;
     const int nx = g.nx, ny = g.ny, nz = g.nz;
-    if (4 * q >= nx || 2 * J >= ny) return;
+    if (!strip_at(nx / 4, ny / 2, flat, q, J)) return;
     const int cnx = nx >> 1, cny = ny >> 1, cnz = nz >> 1, cplane = cnx * cny;
     const bool px = g.per[0] != 0, py = g.per[1] != 0, pz = g.per[2] != 0;
     // coarse x = 2q - 1 and 2q + 2 with their ghost rule; rows J - 1, J + 1 likewise
@@ -1347,15 +1374,15 @@ k_update_residual(const LevelGeom g, double* __restrict__ phi, const float* __re
 // stores of phi and r, the z neighbours carried in registers, the z loop
 // unrolled by two so the next plane's loads overlap the current arithmetic.
 
-template <bool UNIFORM>
+// TWOD: the z term, zero there, is left out.
+template <bool UNIFORM, bool TWOD>
 __global__ void __launch_bounds__(BX * BY, 4)
 k_update_residual4(const LevelGeom g, double* __restrict__ phi, const float* __restrict__ e,
-                   double* __restrict__ r64, float* __restrict__ r32, Partial* partials, int kchunk) {
-    const int q = blockIdx.x * BX + threadIdx.x;        // strip: cells 4q .. 4q + 3
-    const int j = blockIdx.y * BY + threadIdx.y;
+                   double* __restrict__ r64, float* __restrict__ r32, Partial* partials, int kchunk, int flat) {
+    int q, j;                                           // strip: cells 4q .. 4q + 3
     const int nx = g.nx, ny = g.ny, nz = g.nz;
     float sq = 0.0f, mx = 0.0f;
-    if (4 * q < nx && j < ny) {
+    if (strip_at(nx / 4, ny, flat, q, j)) {
         const int i0 = 4 * q, plane = nx * ny;
         const bool px = g.per[0] != 0, py = g.per[1] != 0, pz = g.per[2] != 0;
         const int k0 = blockIdx.z * kchunk;
@@ -1372,10 +1399,10 @@ k_update_residual4(const LevelGeom g, double* __restrict__ phi, const float* __r
             const float xr = i0 + 4 < nx ? e[idx + 4] : (px ? e[idx + 4 - nx] : -c.w);
             double2 ra = ld_d2(r64 + idx), rb = ld_d2(r64 + idx + 2);
             double2 pa = ld_d2(phi + idx), pb = ld_d2(phi + idx + 2);
-            ra.x = update_r<UNIFORM>(g.ihx2, g.ihy2, g.ihz2, c.x, xl, c.y, ym.x, yp.x, zm.x, zp.x, ra.x);
-            ra.y = update_r<UNIFORM>(g.ihx2, g.ihy2, g.ihz2, c.y, c.x, c.z, ym.y, yp.y, zm.y, zp.y, ra.y);
-            rb.x = update_r<UNIFORM>(g.ihx2, g.ihy2, g.ihz2, c.z, c.y, c.w, ym.z, yp.z, zm.z, zp.z, rb.x);
-            rb.y = update_r<UNIFORM>(g.ihx2, g.ihy2, g.ihz2, c.w, c.z, xr, ym.w, yp.w, zm.w, zp.w, rb.y);
+            ra.x = update_r<UNIFORM, TWOD>(g.ihx2, g.ihy2, g.ihz2, c.x, xl, c.y, ym.x, yp.x, zm.x, zp.x, ra.x);
+            ra.y = update_r<UNIFORM, TWOD>(g.ihx2, g.ihy2, g.ihz2, c.y, c.x, c.z, ym.y, yp.y, zm.y, zp.y, ra.y);
+            rb.x = update_r<UNIFORM, TWOD>(g.ihx2, g.ihy2, g.ihz2, c.z, c.y, c.w, ym.z, yp.z, zm.z, zp.z, rb.x);
+            rb.y = update_r<UNIFORM, TWOD>(g.ihx2, g.ihy2, g.ihz2, c.w, c.z, xr, ym.w, yp.w, zm.w, zp.w, rb.y);
             *reinterpret_cast<double2*>(r64 + idx) = ra;
             *reinterpret_cast<double2*>(r64 + idx + 2) = rb;
             pa.x += f2d_bits(c.x);
@@ -1911,53 +1938,7 @@ k_gravity_fx4(const LevelGeom g, const double* __restrict__ u, double* __restric
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kRedThreads) k_finalize(const Partial* __restrict__ p, int n,
                                                           Reduced* out) {
-    // Fixed order (deterministic): thread t folds partials t, t + 256, ...
-    // four at a time so that their loads are in flight together, then the
-    // warps fold by shuffles and warp 0 folds the eight warp results.
-    __shared__ double s_sq[kRedThreads / 32], s_mx[kRedThreads / 32], s_sum[kRedThreads / 32];
-    double sq = 0.0, mx = 0.0, sm = 0.0;
-    int t = threadIdx.x;
-    for (; t + 3 * kRedThreads < n; t += 4 * kRedThreads) {
-        Partial a[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) a[e] = p[t + e * kRedThreads];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            sq += a[e].sumsq;
-            mx = fmax(mx, a[e].maxabs);
-            sm += a[e].sum;
-        }
-    }
-    for (; t < n; t += kRedThreads) {
-        sq += p[t].sumsq;
-        mx = fmax(mx, p[t].maxabs);
-        sm += p[t].sum;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        sq += __shfl_down_sync(0xffffffffu, sq, o);
-        mx = fmax(mx, __shfl_down_sync(0xffffffffu, mx, o));
-        sm += __shfl_down_sync(0xffffffffu, sm, o);
-    }
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) {
-        s_sq[w] = sq;
-        s_mx[w] = mx;
-        s_sum[w] = sm;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double a = s_sq[0], b = s_mx[0], c = s_sum[0];
-        for (int k = 1; k < kRedThreads / 32; ++k) {
-            a += s_sq[k];
-            b = fmax(b, s_mx[k]);
-            c += s_sum[k];
-        }
-        out->sumsq = a;
-        out->maxabs = b;
-        out->sum = c;
-        out->count = double(n);
-    }
+    fold_partials(p, n, out);
 }
 
 template <typename T>
@@ -2187,7 +2168,8 @@ cudaError_t launch_residual_restrict(const LevelGeom& g, const T* u, const T* rh
                                reinterpret_cast<uintptr_t>(coarse_out)) & 15) == 0;
         if (!has_faces(g) && (g.nx & 3) == 0 && (g.ny & 1) == 0 && (g.nz & 1) == 0 && aligned) {
             // as many blocks as the scalar launch at most (the partials buffer)
-            const long long gx = (g.nx / 4 + BX - 1) / BX, gy = (g.ny / 2 + BY - 1) / BY;
+            const StripGrid at(g.nx / 4, g.ny / 2);
+            const long long gx = at.gx, gy = at.gy;
             const long long chunks = std::min<long long>(g.nz / 2, std::max(1LL, restrict_blocks(g) / (gx * gy)));
             int kc = (int)((g.nz + chunks - 1) / chunks);
             kc += kc & 1;
@@ -2196,9 +2178,9 @@ cudaError_t launch_residual_restrict(const LevelGeom& g, const T* u, const T* rh
             while (kc < 16 && gx * gy * ((g.nz + 2 * kc - 1) / (2 * kc)) >= 3LL * sm_count()) kc *= 2;
             dim3 block(BX, BY, 1);
             dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)((g.nz + kc - 1) / kc));
-            if (want == kWantNorms) k_residual_restrict4<kWantNorms><<<grid, block, 0, st>>>(g, u, rhs, coarse_out, partials, kc);
-            else if (want == kWantSum) k_residual_restrict4<kWantSum><<<grid, block, 0, st>>>(g, u, rhs, coarse_out, partials, kc);
-            else k_residual_restrict4<kWantNothing><<<grid, block, 0, st>>>(g, u, rhs, coarse_out, partials, kc);
+            if (want == kWantNorms) k_residual_restrict4<kWantNorms><<<grid, block, 0, st>>>(g, u, rhs, coarse_out, partials, kc, at.flat);
+            else if (want == kWantSum) k_residual_restrict4<kWantSum><<<grid, block, 0, st>>>(g, u, rhs, coarse_out, partials, kc, at.flat);
+            else k_residual_restrict4<kWantNothing><<<grid, block, 0, st>>>(g, u, rhs, coarse_out, partials, kc, at.flat);
             if (nblocks_out) *nblocks_out = (int)(grid.x * grid.y * grid.z);
             return cudaGetLastError();
         }
@@ -2229,13 +2211,14 @@ cudaError_t launch_prolong_correct(const LevelGeom& g, const T* coarse, T* fine_
     if constexpr (std::is_same<T, float>::value) {
         const bool aligned = ((reinterpret_cast<uintptr_t>(coarse) | reinterpret_cast<uintptr_t>(fine_u)) & 15) == 0;
         if ((g.nx & 3) == 0 && (g.ny & 1) == 0 && (g.nz & 1) == 0 && aligned) {
-            const long long gx = (g.nx / 4 + BX - 1) / BX, gy = (g.ny / 2 + BY - 1) / BY;
+            const StripGrid at(g.nx / 4, g.ny / 2);
+            const long long gx = at.gx, gy = at.gy;
             const long long chunks = std::min<long long>(g.nz / 2, std::max(1LL, 16LL * 152 / (gx * gy)));
             int kc = (int)((g.nz + chunks - 1) / chunks);
             kc += kc & 1;
             dim3 block(BX, BY, 1);
             dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)((g.nz + kc - 1) / kc));
-            k_prolong_correct4<<<grid, block, 0, st>>>(g, coarse, fine_u, kc);
+            k_prolong_correct4<<<grid, block, 0, st>>>(g, coarse, fine_u, kc, at.flat);
             return cudaGetLastError();
         }
     }
@@ -2252,14 +2235,32 @@ cudaError_t launch_update_residual(const LevelGeom& g, double* phi, const float*
     const bool aligned = ((reinterpret_cast<uintptr_t>(phi) | reinterpret_cast<uintptr_t>(e) |
                            reinterpret_cast<uintptr_t>(r64) | reinterpret_cast<uintptr_t>(r32)) & 15) == 0;
     if ((g.nx & 3) == 0 && aligned) {
-        // as many blocks as the scalar residual launch at most (the partials buffer)
-        const long long gx = (g.nx / 4 + BX - 1) / BX, gy = (g.ny + BY - 1) / BY;
-        const long long chunks = std::min<long long>(g.nz, std::max(1LL, residual_blocks(g) / (gx * gy)));
+        // (as many blocks as the scalar residual launch at most: the partials buffer)
+        const StripGrid at(g.nx / 4, g.ny);
+        const long long gx = at.gx, gy = at.gy;
+        // z chunks that fill one wave of four blocks per SM, or up to three waves where
+        // that leaves fewer slots idle: solves with one wave against as many blocks as
+        // the scalar launch: 112 x 80 x 144 2154 and 2100 us, 128^3 2832 and 2785, GS-RB
+        // 192^3 2329 and 2297, 64 uneven grids 46.7 and 45.4 ms (half a wave: 2142, 2819,
+        // 2425 us, 45.2 ms)
+        const long long slots = 4 * sm_count(), most = std::max(1LL, residual_blocks(g) / (gx * gy));
+        long long chunks = 1;
+        double fill = -1.0;
+        for (int w = 1; w <= 3; ++w) {
+            const long long c = std::min<long long>({(long long)g.nz, most, std::max(1LL, w * slots / (gx * gy))});
+            const long long blocks = gx * gy * c, waves = (blocks + slots - 1) / slots;
+            const double x = double(blocks) / double(waves * slots);
+            if (x > fill + 0.05) {
+                fill = x;
+                chunks = c;
+            }
+        }
         const int kc = (int)((g.nz + chunks - 1) / chunks);
         dim3 block(BX, BY, 1);
         dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)((g.nz + kc - 1) / kc));
-        if (uniform4) k_update_residual4<true><<<grid, block, 0, st>>>(g, phi, e, r64, r32, partials, kc);
-        else k_update_residual4<false><<<grid, block, 0, st>>>(g, phi, e, r64, r32, partials, kc);
+        if (g.twod) k_update_residual4<false, true><<<grid, block, 0, st>>>(g, phi, e, r64, r32, partials, kc, at.flat);
+        else if (uniform4) k_update_residual4<true, false><<<grid, block, 0, st>>>(g, phi, e, r64, r32, partials, kc, at.flat);
+        else k_update_residual4<false, false><<<grid, block, 0, st>>>(g, phi, e, r64, r32, partials, kc, at.flat);
         if (nblocks_out) *nblocks_out = (int)(grid.x * grid.y * grid.z);
         return cudaGetLastError();
     }

@@ -834,8 +834,9 @@ sg_status vcycle(sg_grid* g, int L, W* u0, const W* rhs0, bool faces, bool zero0
     return SG_OK;
 }
 
-// Residual norm of (phi, f) at level 0 into red[0]; mixed mode also writes r32.
-sg_status level0_residual(sg_grid* g, const double* phi, const double* f, bool faces) {
+// Residual norm of (phi, f) at level 0 into red[0]; mixed mode also writes r32.  nb_out:
+// the norm is left in that many block partials.
+sg_status level0_residual(sg_grid* g, const double* phi, const double* f, bool faces, int* nb_out = nullptr) {
     int nb = 0, nk = 1;
     const LevelGeom G = geom(g, 0, faces);
     {
@@ -846,8 +847,13 @@ sg_status level0_residual(sg_grid* g, const double* phi, const double* f, bool f
     else
         SG_CK(launch_residual<double, double>(G, phi, f, (double*)nullptr, g->partials, &nb, g->st));
     }
+    g->launches += nk;
+    if (nb_out) {
+        *nb_out = nb;
+        return SG_OK;
+    }
     SG_CK(launch_finalize(g->partials, nb, g->red, g->st));
-    g->launches += nk + 1;
+    ++g->launches;
     return SG_OK;
 }
 
@@ -869,8 +875,9 @@ sg_status level0_residual_zero(sg_grid* g, const double* f, bool faces) {
 
 // Everything one cycle enqueues after the first residual: V-cycle, update,
 // residual + norm, and the copies of the norm / coarse count to pinned memory.
-// One V-cycle and the residual norm after it (into red[0]); no host copies.
-sg_status cycle_core(sg_grid* g, int L, double* phi, const double* f, bool faces) {
+// One V-cycle and the residual norm after it (into red[0], or left in *nb_out block
+// partials); no host copies.
+sg_status cycle_core(sg_grid* g, int L, double* phi, const double* f, bool faces, int* nb_out = nullptr) {
     if (g->precision == SG_MIXED) {
         // the inner cycle starts from e = 0: its first super-step takes Y0 = 0
         float* e = (float*)g->lv[0].u;
@@ -883,11 +890,16 @@ sg_status cycle_core(sg_grid* g, int L, double* phi, const double* f, bool faces
             SG_CK(launch_update_residual(geom(g, 0, false), phi, e_final, g->r64, (float*)g->lv[0].rhs,
                                          g->partials, &nb, g->st));
         }
-        SG_CK(launch_finalize(g->partials, nb, g->red, g->st));
-        g->launches += 2;
+        ++g->launches;
+        if (nb_out) {
+            *nb_out = nb;
+        } else {
+            SG_CK(launch_finalize(g->partials, nb, g->red, g->st));
+            ++g->launches;
+        }
     } else {
         SG_TRY(vcycle<double>(g, L, phi, f, faces, false, nullptr));
-        SG_TRY(level0_residual(g, phi, f, faces));
+        SG_TRY(level0_residual(g, phi, f, faces, nb_out));
     }
     return SG_OK;
 }
@@ -1195,7 +1207,7 @@ sg_status solve_end(sg_grid* g, SolveState& S, sg_solve_info* info) {
 // edge (a batch adds one branch per grid):
 //   init -> WHILE(outer) { WHILE(inner) { V-cycle, residual norm, step }
 //                          [mixed: the true FP64 residual]  confirm }
-// The one-thread init / step / confirm kernels (kernels_loop.cu) take the host
+// The one-block init / step / confirm kernels (kernels_loop.cu) take the host
 // loop's decisions on the device and set the two conditions.  *per_cycle and
 // *per_confirm receive the kernels of one inner and one outer iteration.
 sg_status add_solve_loop(sg_grid* g, cudaGraph_t graph, int L, double* phi, const double* f, bool faces,
@@ -1249,16 +1261,18 @@ sg_status add_solve_loop(sg_grid* g, cudaGraph_t graph, int L, double* phi, cons
         if (resident) SG_CK(launch_tail<float>(tail, g->twod, tail_launch, st));
         else SG_TRY(add_while(hi, &inner_body));
         const long long b0 = g->launches;
-        if (g->precision == SG_MIXED) SG_TRY(level0_residual(g, phi, f, faces));
-        SG_CK(launch_loop_confirm(g->dloop, g->red, ho, hi, !resident, st));
+        int nb = 0;
+        if (g->precision == SG_MIXED) SG_TRY(level0_residual(g, phi, f, faces, &nb));
+        SG_CK(launch_loop_confirm(g->dloop, g->partials, nb, g->red, ho, hi, !resident, st));
         *per_confirm = g->launches - b0 + (resident ? 2 : 1);
         return SG_OK;
     }));
     *per_cycle = 0;
     if (!resident) SG_TRY(capture(inner_body, [&]() -> sg_status {
         const long long b0 = g->launches;
-        SG_TRY(cycle_core(g, L, phi, f, faces));
-        SG_CK(launch_loop_step(g->dloop, g->red, g->d_ss, g->d_sched, hi, st));
+        int nb = 0;
+        SG_TRY(cycle_core(g, L, phi, f, faces, &nb));
+        SG_CK(launch_loop_step(g->dloop, g->partials, nb, g->red, g->d_ss, g->d_sched, hi, st));
         *per_cycle = g->launches - b0 + 1;
         return SG_OK;
     }));

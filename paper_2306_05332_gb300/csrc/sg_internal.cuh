@@ -170,10 +170,12 @@ struct DeviceLoop : LoopState {
 // has_inner false: the inner loop is no WHILE node (the resident solve runs it in one launch)
 cudaError_t launch_loop_init(const DeviceLoop* d, cudaGraphConditionalHandle outer, cudaGraphConditionalHandle inner,
                              bool has_inner, cudaStream_t st);
-cudaError_t launch_loop_step(DeviceLoop* d, const Reduced* red, const int* ss_done, const int* sched,
-                             cudaGraphConditionalHandle inner, cudaStream_t st);
-cudaError_t launch_loop_confirm(DeviceLoop* d, const Reduced* red, cudaGraphConditionalHandle outer,
-                                cudaGraphConditionalHandle inner, bool has_inner, cudaStream_t st);
+// partials, nb: the residual's block partials, folded into *red first (confirm: none where nb = 0)
+cudaError_t launch_loop_step(DeviceLoop* d, const Partial* partials, int nb, Reduced* red, const int* ss_done,
+                             const int* sched, cudaGraphConditionalHandle inner, cudaStream_t st);
+cudaError_t launch_loop_confirm(DeviceLoop* d, const Partial* partials, int nb, Reduced* red,
+                                cudaGraphConditionalHandle outer, cudaGraphConditionalHandle inner, bool has_inner,
+                                cudaStream_t st);
 // The decision after a cycle with relative residual rel and largest residual maxabs, on
 // the counters of d: true to run another.  *record: the residual goes into the history.
 __device__ __forceinline__ bool loop_decide(LoopState& d, double rel, double maxabs, bool* record) {

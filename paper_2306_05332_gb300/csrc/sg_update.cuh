@@ -35,8 +35,8 @@ __device__ __forceinline__ float d2f_bits(double x) {
 // r -= (A_0 e) for one cell, A_0 the homogeneous operator, formed without
 // rounding: the FP32 neighbour sum is split by TwoSum into a value and its
 // exact error (products by -6 and -2 are exact up to one FMA term), and both
-// enter r through FP64 FMAs.
-template <bool UNIFORM>
+// enter r through FP64 FMAs.  TWOD: without the z axis (its 1 / h^2 is zero).
+template <bool UNIFORM, bool TWOD = false>
 __device__ __forceinline__ double update_r(double ihx2, double ihy2, double ihz2, float c, float xm, float xp,
                                            float ym, float yp, float zm, float zp, double r) {
     if (UNIFORM) {
@@ -59,7 +59,7 @@ __device__ __forceinline__ double update_r(double ihx2, double ihy2, double ihz2
         const float a[3][2] = {{xm, xp}, {ym, yp}, {zm, zp}};
         const double ih[3] = {ihx2, ihy2, ihz2};
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
+        for (int d = 0; d < (TWOD ? 2 : 3); ++d) {
             float s, comp, t;
             two_sum(a[d][0], a[d][1], s, comp);
             two_sum(s, m2, s, t);
