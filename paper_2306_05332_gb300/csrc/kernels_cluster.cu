@@ -879,15 +879,11 @@ int row_stride(int nx, bool twod) {
 }  // namespace
 
 cudaError_t tail_configure() {
-    static bool configured = false;              // (the caller holds a lock)
-    if (configured) return cudaSuccess;
     cudaError_t e;
     if ((e = configure_one<float, false>()) != cudaSuccess) return e;
     if ((e = configure_one<float, true>()) != cudaSuccess) return e;
     if ((e = configure_one<double, false>()) != cudaSuccess) return e;
-    if ((e = configure_one<double, true>()) != cudaSuccess) return e;
-    configured = true;
-    return cudaSuccess;
+    return configure_one<double, true>();
 }
 
 // Layout of levels lv[0 .. nl) (nx, ny, nz set; two-dimensional ones as nx x 1 x ny)

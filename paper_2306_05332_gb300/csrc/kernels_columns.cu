@@ -327,6 +327,16 @@ cudaError_t columns_configure() {
     return col_configure<3, true>();
 }
 
+// (by the attribute that columns_configure sets last)
+bool columns_configured() {
+    cudaFuncAttributes a;
+    if (cudaFuncGetAttributes(&a, k_superstep_columns<3, true, false>) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.maxDynamicSharedSizeBytes == (int)Col<3, true>::BYTES;
+}
+
 cudaError_t launch_superstep_columns(const LevelGeom& g, int order, int s, bool zero_y0, const FusedCoef& cf,
                                      const float* y0, const float* f, float* out, cudaStream_t st) {
     const ColCoef k = col_coef(make_lean_coef(g, order, s, cf), zero_y0);

@@ -400,7 +400,6 @@ cudaError_t fused_configure() {
     int dev = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = columns_configure()) != cudaSuccess) return e;    // s = 2, 3 (kernels_columns.cu)
     if ((e = lean_configure()) != cudaSuccess) return e;       // s = 2, 3 on request (kernels_superstep.cu)
     if ((e = configure_s<4>()) != cudaSuccess) return e;
     if ((e = configure_s<5>()) != cudaSuccess) return e;

@@ -1539,13 +1539,16 @@ sg_status create_grid(int nx, int ny, int nz, const double lo[3], const double h
                       int precision, void* cuda_stream, sg_grid** out, bool twod) {
     const int n[3] = {nx, ny, nz};
     {
-        // one-time kernel attributes and occupancy figures, set by whichever
-        // thread creates a grid first
+        // kernel attributes and occupancy figures, set by whichever thread creates
+        // the first grid of a device's context (about a hundred driver calls)
         static std::mutex configure_mu;
         std::lock_guard<std::mutex> lock(configure_mu);
-        SG_CK(coarse_configure());
-        SG_CK(fused_configure());
-        SG_CK(tail_configure());
+        if (!columns_configured()) {
+            SG_CK(coarse_configure());
+            SG_CK(fused_configure());
+            SG_CK(tail_configure());
+            SG_CK(columns_configure());
+        }
     }
     sg_grid* g = new sg_grid();
     static std::atomic<unsigned long long> serials{0};

@@ -222,6 +222,7 @@ cudaError_t launch_superstep_lean(const LevelGeom& g, int order, int s, bool zer
                                   bool tma);
 // s = 2, 3: one thread per column (kernels_columns.cu).
 cudaError_t columns_configure();
+bool columns_configured();              // columns_configure has run in the current device's context
 cudaError_t launch_superstep_columns(const LevelGeom& g, int order, int s, bool zero_y0, const FusedCoef& cf,
                                      const float* y0, const float* f, float* out, cudaStream_t st);
 // Launches of the TMA path that gave up a bounded wait (or found their shared
