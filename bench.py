@@ -454,7 +454,7 @@ def run_ours(a, world, rank, local):
     # INFLIGHT independent solves of the workload at a time: one grid per
     # stream, each driven by its own host thread (the library's calls release
     # the interpreter lock); the solves fill each other's idle SMs (small
-    # coarse-level kernels, the one-cluster launch, the one-thread loop kernels)
+    # coarse-level kernels, the one-cluster launch, the one-block loop kernels)
     streams = [stream] + [torch.cuda.Stream(dev) for _ in range(INFLIGHT - 1)]
     grids = [g]
     for st in streams[1:]:
@@ -775,7 +775,7 @@ def run_ours(a, world, rank, local):
                                   "autotuned_max_cycles": max(i["cycles"] for i in tinfo),
                                   "autotuned_max_rel_residual": max(i["rel_residual"] for i in tinfo),
                                   "structure": "one CUDA graph launch per batch: a branch per instance, each "
-                                               "a WHILE loop of V-cycles whose condition a one-thread kernel "
+                                               "a WHILE loop of V-cycles whose condition a one-block kernel "
                                                "sets from the residual on the device"}
         del grids, rhos
 

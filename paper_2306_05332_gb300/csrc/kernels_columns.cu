@@ -13,14 +13,14 @@
 // per stage and phase, double-buffered, so that one barrier a phase is enough.  The
 // halo shrinks by a cell per stage; what a thread computes past it is not used.
 //
-// What bounds it.  The shared-memory pipe (60 wavefronts per warp and phase, 57% of its
-// rate at 256^3) and the issue of its bursts after each barrier; 148 instructions per
-// warp and phase, 76 of them arithmetic.  HBM (Y0, f and Y_s once: 30 us at 256^3) is not.
+// What bounds it.  The shared-memory pipe (about 52 wavefronts per warp and phase) and the
+// issue of its bursts after each barrier; HBM (Y0, f and Y_s once: 30 us at 256^3) is not.
 // One general s = 3 super-step, one stage per thread (k_superstep_lean) and here: 512^3
-// 831 and 483 us, 256^3 119 and 82, 192^3 59 and 41, 128^3 28 and 22 (cold L2); Y0 = 0:
+// 831 and 417 us, 256^3 119 and 70, 192^3 59 and 39, 128^3 28 and 20 (cold L2); Y0 = 0:
 // 256^3 70 and 47 us.  What gave how much at 256^3: this split 96 us; constant ring
 // slots and buffer halves (phases unrolled by six), coefficients as pairs in the
-// constant bank and reflected strips copied like any other 82.  Row pairs per thread
+// constant bank and reflected strips copied like any other 82; f, which no neighbour
+// reads, loaded into registers a phase ahead 70.  Row pairs per thread
 // (384 threads of 158 registers: fewer wavefronts, too few warps) 94 us, 512 threads
 // 100, end cells by shuffles 104.
 #include "sg_superstep.cuh"
@@ -36,10 +36,10 @@ namespace {
 constexpr int kColThreads = 640;        // 20 warps of up to 96 registers
 constexpr int kColRing = 6;             // planes of the copy ring: four in flight ahead of the phase's own
 
-template <int S, bool ZERO>
+template <int S, bool ZERO, bool VEC>
 struct Col {
     static constexpr int NS = ZERO ? S - 1 : S;          // stencil stages (Y0 = 0: stage 1 is a multiple of f)
-    static constexpr int NF = ZERO ? 1 : 2;              // staged fields: Y0 and f, or f
+    static constexpr int NF = ZERO || VEC ? 1 : 2;       // staged fields: f; Y0 (VEC: f goes to registers); Y0 and f
     static constexpr int STRIP = 4 * kColThreads;        // floats of one field's strips
     static constexpr int SLOT = NF * STRIP;
     static constexpr int OE = kColRing * SLOT;           // end cells of the staged plane: 2 x (x, w)
@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(kColThreads, 1)
 k_superstep_columns(const __grid_constant__ LevelGeom g, const __grid_constant__ ColCoef k,
                     const __grid_constant__ ColPlan p, const float* __restrict__ y0g, const float* __restrict__ fg,
                     float* __restrict__ outg) {
-    using C = Col<S, ZERO>;
+    using C = Col<S, ZERO, VEC>;
     constexpr int NS = C::NS, R = kColRing;
     extern __shared__ __align__(128) float sm[];
     const int tid = threadIdx.x;
@@ -117,8 +117,7 @@ k_superstep_columns(const __grid_constant__ LevelGeom g, const __grid_constant__
         float* dst = sm + slot * C::SLOT;
         if constexpr (VEC) {
             if (some) {
-                if constexpr (!ZERO) cpa16(dst + 4 * tid, y0g + (src + off));
-                cpa16(dst + (C::NF - 1) * C::STRIP + 4 * tid, fg + (src + off));
+                cpa16(dst + 4 * tid, (ZERO ? fg : y0g) + (src + off));
             }
         } else {
             if constexpr (!ZERO) issue(ld, dst, y0g + src);
@@ -145,6 +144,8 @@ k_superstep_columns(const __grid_constant__ LevelGeom g, const __grid_constant__
         w_end[ends + kColThreads] = v.w;
     };
 
+    float4 f_next = zero4;
+    bool ng_before = false;
     // Phase u, u % 6 = U: the z windows, the W fields, the ring slots and the halves of the
     // buffers rotate by constants (a: the staged field, b and c: the outputs of the first two
     // stencil stages)
@@ -158,19 +159,22 @@ k_superstep_columns(const __grid_constant__ LevelGeom g, const __grid_constant__
         // plane t has landed (this thread's copies): turn its reflected cells
         asm volatile("cp.async.wait_group %0;\n" ::"n"(kColRing - 3) : "memory");
         int zsign = 1;
-        if (!pz && (unsigned)(t0 + u) >= (unsigned)nz) map_axis(t0 + u, nz, false, &zsign);
+        const int zt = map_axis(t0 + u, nz, pz, &zsign);
         a_up = ld4(s_own + now);
+        [[maybe_unused]] float4 f = f_next;         // f of plane t - 1, loaded a phase ago
         if constexpr (VEC) {
+            if (!ZERO && some) f_next = __ldg(reinterpret_cast<const float4*>(fg + (zt * plane + off)));
+            auto turn = [&](float4 v, bool ng) {
+                if (rev) v = make_float4(v.w, v.z, v.y, v.x);
+                return ng ? make_float4(-v.x, -v.y, -v.z, -v.w) : v;
+            };
             const bool ng = neg != (zsign < 0);
+            if (!ZERO && (rev || ng_before)) f = turn(f, ng_before);
             if (rev || ng) {
-                auto turn = [&](float4 v) {
-                    if (rev) v = make_float4(v.w, v.z, v.y, v.x);
-                    return ng ? make_float4(-v.x, -v.y, -v.z, -v.w) : v;
-                };
-                a_up = turn(a_up);
+                a_up = turn(a_up, ng);
                 st4(w_own + now, a_up);
-                if constexpr (!ZERO) st4(w_own + now + C::STRIP, turn(ld4(s_own + now + C::STRIP)));
             }
+            ng_before = ng;
         } else {
             fixup(ld, sm + now, zsign);
             if constexpr (!ZERO) fixup(ld, sm + now + C::STRIP, zsign);
@@ -188,7 +192,7 @@ k_superstep_columns(const __grid_constant__ LevelGeom g, const __grid_constant__
                                 scale4(k.kz3, a_dn));
             }
         } else {
-            const float4 f = ld4(s_own + before + C::STRIP);
+            if constexpr (!VEC) f = ld4(s_own + before + C::STRIP);
             first_strip<S>(k.first, a_cn, e1.n, e1.s, a_dn, a_up, e1.l, e1.r, f, b_up, w2w, w3w);
             const Nb e2 = around(yb, yb + C::STRIP);
             v = later_strip(b_cn, e2.n, e2.s, b_dn, b_up, e2.l, e2.r, k.ax[0], k.ay[0], k.az[0], k.b[0], w2r);
@@ -296,22 +300,21 @@ ColCoef col_coef(const LeanCoef& k, bool zero) {
 template <int S, bool ZERO>
 cudaError_t col_run(const LevelGeom& g, const ColCoef& k, const float* y0, const float* f, float* out,
                     cudaStream_t st) {
-    using C = Col<S, ZERO>;
+    using C = Col<S, ZERO, false>;
     const bool aligned = ((reinterpret_cast<uintptr_t>(y0) | reinterpret_cast<uintptr_t>(f) |
                            reinterpret_cast<uintptr_t>(out)) & 15) == 0;
     const ColPlan p = col_plan(g, C::NS);
     const unsigned grid = (unsigned)(p.tiles_x * p.tiles_y * p.chunks);
-    if ((g.nx & 3) == 0 && aligned) k_superstep_columns<S, ZERO, true><<<grid, p.threads, C::BYTES, st>>>(g, k, p, y0, f, out);
+    if ((g.nx & 3) == 0 && aligned) k_superstep_columns<S, ZERO, true><<<grid, p.threads, Col<S, ZERO, true>::BYTES, st>>>(g, k, p, y0, f, out);
     else k_superstep_columns<S, ZERO, false><<<grid, p.threads, C::BYTES, st>>>(g, k, p, y0, f, out);
     return cudaGetLastError();
 }
 
 template <int S, bool ZERO>
 cudaError_t col_configure() {
-    const int bytes = (int)Col<S, ZERO>::BYTES;
     const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    const cudaError_t e = cudaFuncSetAttribute(k_superstep_columns<S, ZERO, true>, attr, bytes);
-    return e != cudaSuccess ? e : cudaFuncSetAttribute(k_superstep_columns<S, ZERO, false>, attr, bytes);
+    const cudaError_t e = cudaFuncSetAttribute(k_superstep_columns<S, ZERO, true>, attr, (int)Col<S, ZERO, true>::BYTES);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(k_superstep_columns<S, ZERO, false>, attr, (int)Col<S, ZERO, false>::BYTES);
 }
 
 }  // namespace
@@ -334,7 +337,7 @@ bool columns_configured() {
         cudaGetLastError();
         return false;
     }
-    return a.maxDynamicSharedSizeBytes == (int)Col<3, true>::BYTES;
+    return a.maxDynamicSharedSizeBytes == (int)Col<3, true, false>::BYTES;
 }
 
 cudaError_t launch_superstep_columns(const LevelGeom& g, int order, int s, bool zero_y0, const FusedCoef& cf,
