@@ -62,10 +62,9 @@ SOLVER = dict(rkl_order=2, s_smooth=3, tau_frac=0.9, n_pre=5, n_post=3, inner_n_
               coarse_tol=1e-2, coarse_max_ss=64)
 METRIC = "Poisson solves/s to rel. residual 1e-8 at 256^3"
 FALLBACK_HBM_GBS = 6800.0
-# FP64 instructions per cell and stage of the FP64 stage kernel, averaged over
-# an s = 3 RKL2 super-step (one first stage, 13.5; two later ones, 16.5), as
-# counted by ncu (smsp__inst_executed_pipe_fp64) on 256^3 launches
-FP64_INSTR_PER_STAGE_CELL = 15.5
+# FP64 operations per cell and stage of the FP64 stage kernel where h is the same on
+# every axis, averaged over an s = 3 RKL2 super-step (9, 12 and 13 in its stages)
+FP64_INSTR_PER_STAGE_CELL = 34.0 / 3.0
 
 
 def args_():
@@ -631,9 +630,8 @@ def run_ours(a, world, rank, local):
         i64 = g64.solve(tol=TOL, levels=LEVELS)
         t64 = (time.perf_counter() - t0) * 1e3
         # its roofline: the level-0 stage kernels are bound by the FP64 pipe, not
-        # HBM; FP64 instructions per cell counted by ncu on these kernels
-        # (13.5 in a first stage, 16.5 in a later one: 15.5 on average over an
-        # s = 3 super-step), against this GPU's measured FP64 FMA rate
+        # HBM: the kernel's FP64 operations per cell against this GPU's measured
+        # FP64 FMA rate
         fp64_tflops, _ = sg.measure_fp64_rate()
         g64.set_density(rho_dev, 1.0)
         g64.set_profiling(True)
