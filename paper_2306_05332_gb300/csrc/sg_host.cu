@@ -260,6 +260,7 @@ struct sg_grid {
     Reduced* host_red = nullptr;    // pinned mirror
     int* d_sched = nullptr;
     int sched_cap = 0;
+    std::vector<int> sched;         // the schedule d_sched holds
     int* d_ss = nullptr;            // coarse super-steps done (device)
     unsigned* d_mexp = nullptr;     // the exact residual's fixed-point scale (device)
     int* host_ss = nullptr;         // pinned mirror
@@ -432,6 +433,8 @@ sg_status check_opts(const sg_options* o) {
 }
 
 sg_status ensure_sched(sg_grid* g, const std::vector<int>& s) {
+    if (g->sched == s) return SG_OK;            // on the device already
+    g->sched.clear();
     if ((int)s.size() > g->sched_cap) {
         if (g->d_sched) cudaFree(g->d_sched);
         g->d_sched = nullptr;
@@ -440,6 +443,7 @@ sg_status ensure_sched(sg_grid* g, const std::vector<int>& s) {
     }
     SG_CK(cudaMemcpyAsync(g->d_sched, s.data(), s.size() * sizeof(int), cudaMemcpyHostToDevice, g->st));
     SG_CK(cudaStreamSynchronize(g->st));
+    g->sched = s;
     return SG_OK;
 }
 
@@ -1024,7 +1028,9 @@ struct SolveState {
 
 // r0 = ||L 0 - f|| (boundary contribution of phi = 0 included), the first
 // residual, the coarse schedule; leaves the residual of the start in host_red[0].
-sg_status solve_begin(sg_grid* g, SolveState& S, double tol, int L, double* phi, const double* f, bool faces,
+// In two parts, what goes to the stream and what follows once it is done, so that a
+// batch waits once for the starts of all its grids.
+sg_status solve_begin_enqueue(sg_grid* g, SolveState& S, double tol, int L, double* phi, const double* f, bool faces,
                       bool have_guess) {
     if (g->opt.smoother == SG_SMOOTH_GSRB) {
         // red-black colouring must hold across a periodic wrap on every swept level
@@ -1058,6 +1064,12 @@ sg_status solve_begin(sg_grid* g, SolveState& S, double tol, int L, double* phi,
         SG_TRY(level0_residual(g, phi, f, faces));
     }
     SG_CK(cudaMemcpyAsync(g->host_red, g->red, sizeof(Reduced), cudaMemcpyDeviceToHost, g->st));
+    return SG_OK;
+}
+
+sg_status solve_begin_finish(sg_grid* g, SolveState& S, bool have_guess) {
+    const int L = S.L;
+    const Level& L0 = g->lv[0];
     SG_CK(cudaStreamSynchronize(g->st));
     prof_sync_point(g, false);
     S.nn = double(L0.n);
@@ -1081,6 +1093,12 @@ sg_status solve_begin(sg_grid* g, SolveState& S, double tol, int L, double* phi,
     S.done = false;
     S.status = SG_OK;
     return SG_OK;
+}
+
+sg_status solve_begin(sg_grid* g, SolveState& S, double tol, int L, double* phi, const double* f, bool faces,
+                      bool have_guess) {
+    SG_TRY(solve_begin_enqueue(g, S, tol, L, phi, f, faces, have_guess));
+    return solve_begin_finish(g, S, have_guess);
 }
 
 // Record the residual now in host_red[0]; decide whether the solve is over.
@@ -1899,7 +1917,15 @@ sg_status sg_solve_batch(sg_grid* const* grids, int n, double tol, sg_solve_info
     std::vector<SolveState> S(P);
     for (size_t k = 0; k < P; ++k) {
         sg_grid* g = grids[par[k]];
-        SG_TRY(solve_begin(g, S[k], tol, g->max_levels, g->phi, g->f, g->have_faces, g->guess_set));
+        const sg_status st = solve_begin_enqueue(g, S[k], tol, g->max_levels, g->phi, g->f, g->have_faces, g->guess_set);
+        if (st != SG_OK) {                      // the starts before it are left complete
+            for (size_t q = 0; q <= k; ++q) cudaStreamSynchronize(grids[par[q]]->st);
+            return st;
+        }
+    }
+    for (size_t k = 0; k < P; ++k) {
+        sg_grid* g = grids[par[k]];
+        SG_TRY(solve_begin_finish(g, S[k], g->guess_set));
         g->guess_set = false;
         SG_TRY(solve_check(g, S[k]));
     }
