@@ -63,7 +63,7 @@ namespace sg {
 namespace {
 
 constexpr int kTailMaxNC = 16;           // CTAs per cluster (16: a non-portable size, where the device allows it)
-constexpr size_t kSmemLimit = 227u * 1024u - 6144u;   // dynamic shared memory per CTA, next to the static tables
+constexpr size_t kSmemLimit = 227u * 1024u - 5120u;   // dynamic shared memory per CTA, next to the static tables
 constexpr int kMuTable = 128;            // entries of the table of mu_j of the coarse solve
 constexpr int kSchedTable = 64;          // entries of its schedule kept in shared memory
 
@@ -87,6 +87,10 @@ __device__ __forceinline__ V fma2(T a, V b, V c) {
 template <typename T, typename V>
 __device__ __forceinline__ V mul2(T a, V b) {
     return mk2(a * b.x, a * b.y);
+}
+template <typename V>
+__device__ __forceinline__ V add2(V a, V b) {
+    return mk2(a.x + b.x, a.y + b.y);
 }
 template <typename V>
 __device__ __forceinline__ V neg2(V v) {
@@ -271,7 +275,7 @@ __global__ void __launch_bounds__(tail_threads<T>()) k_tail_levels(const __grid_
     // the parameter bank in every stage and at every change of level cost more than
     // the arithmetic between them (a stage of a 4^3 level, 16 threads: 795 cycles)
     __shared__ TailLevel<T> lvs[kTailMaxLevels];
-    __shared__ T coef[kTailMaxS + 1][8];         // mu, nu, mu~, c0, gamma~ of stage j; the first: 1, 0, mu~_1, 0, 0
+    __shared__ T coef[kTailMaxS + 1][4];         // mu, nu, c0 of stage j; the first: 1, 0, 0
     __shared__ LoopState state;
     __shared__ double inv_nn, inv_rden;
     // ghost planes arrive on these, exchange n on barrier n & 1 (a neighbour is at most
@@ -297,9 +301,14 @@ __global__ void __launch_bounds__(tail_threads<T>()) k_tail_levels(const __grid_
     for (int j = 1 + tid; j <= p.s; j += blockDim.x) {
         coef[j][0] = j == 1 ? T(1) : p.mu[j];
         coef[j][1] = j == 1 ? T(0) : p.nu[j];
-        coef[j][2] = j == 1 ? p.mut1 : p.mut[j];
-        coef[j][3] = j == 1 || p.order == 1 ? T(0) : p.c0[j];
-        coef[j][4] = j == 1 || p.order == 1 ? T(0) : p.gt[j];
+        coef[j][2] = j == 1 || p.order == 1 ? T(0) : p.c0[j];
+    }
+    // mu~ tau and gamma~ tau of every level but the coarsest, the product in 64 bits
+    for (int n = tid; n < (p.nl - 1) * p.s; n += blockDim.x) {
+        const int l = n / p.s, j = n - l * p.s + 1;
+        const double tau = p.lv[l].tau;
+        reinterpret_cast<V*>(sm + p.lv[l].scaled)[j - 1] =
+            mk2(T(p.mut[j] * tau), j == 1 || p.order == 1 ? T(0) : T(p.gt[j] * tau));
     }
     cl.sync();                                   // every CTA runs before a peer writes into it
 
@@ -324,18 +333,22 @@ __global__ void __launch_bounds__(tail_threads<T>()) k_tail_levels(const __grid_
     auto ld = [](const T* a) { return *reinterpret_cast<const V*>(a); };
     auto st = [](T* a, V v) { *reinterpret_cast<V*>(a) = v; };
 
-    // L c - f of the thread's cells c from buffer y: h_x (x neighbours) + h_y (y
-    // neighbours) + h_z (z neighbours) - 2 (h_x + h_y + h_z) c - f, with nf = -f
+    // L c - f of the thread's cells c from buffer y, nf = -f, by the second differences
+    // (lower - 2 c) + upper of each axis.  (Neighbours summed against one term
+    // -2 (h_x + h_y + h_z) c take two operations a cell less, but the rounding of that
+    // coefficient acts on c itself and not on its differences: one V-cycle of a smooth
+    // 48 x 64 x 56 field was off by 5.0 - 7.1e-7 with it, by 1.2 - 2.1e-7 level by level.)
     auto lap = [&](const H& h, const T* y, const V (&c)[2], const V (&nf)[2], V (&out)[2]) {
 #pragma unroll
         for (int a = 0; a < 2; ++a) {
             const int at = a * h.plane;
             const T xl = y[h.oxl + at], xr = y[h.oxr + at];
-            const V sx = mk2(fmat(h.sxl, xl, c[a].y), fmat(h.sxr, xr, c[a].x));
-            const V sz = a == 0 ? fma2(h.szm, ld(y + h.ozm), c[1]) : fma2(h.szp, ld(y + h.ozp), c[0]);
-            V v = fma2(h.hz, sz, fma2(h.md, c[a], nf[a]));
-            if constexpr (!TWOD) v = fma2(h.hy, fma2(h.sym, ld(y + h.oym + at), mul2(h.syp, ld(y + h.oyp + at))), v);
-            out[a] = fma2(h.hx, sx, v);
+            const V m2 = mul2(T(-2), c[a]);
+            const V dx = mk2(fmat(h.sxl, xl, m2.x) + c[a].y, fmat(h.sxr, xr, m2.y) + c[a].x);
+            const V dz = add2(a == 0 ? fma2(h.szm, ld(y + h.ozm), m2) : fma2(h.szp, ld(y + h.ozp), m2), c[1 - a]);
+            V v = fma2(h.hz, dz, nf[a]);
+            if constexpr (!TWOD) v = fma2(h.hy, fma2(h.syp, ld(y + h.oyp + at), fma2(h.sym, ld(y + h.oym + at), m2)), v);
+            out[a] = fma2(h.hx, dx, v);
         }
     };
     // The cells into buffer `off` of this CTA and, on a split level, the slab's faces
@@ -437,13 +450,14 @@ __global__ void __launch_bounds__(tail_threads<T>()) k_tail_levels(const __grid_
             cur = off == L.buf ? 0 : 1;
             return;
         }
-        const T tau = L.tau;
+        const V* const scaled = reinterpret_cast<const V*>(sm + L.scaled) - 1;
         V y0[2], z[2], m2[2];
         y0[0] = y0[1] = z[0] = z[1] = m2[0] = m2[1] = mk2(T(0), T(0));
         int js = 1;
 #pragma unroll 1
         for (int n = p.s * count; n > 0; --n) {
-            const T mu = coef[js][0], nu = coef[js][1], mt = coef[js][2] * tau, c0 = coef[js][3], gt = coef[js][4] * tau;
+            const T mu = coef[js][0], nu = coef[js][1], c0 = coef[js][2];
+            const V mt_gt = scaled[js];
             V l[2];
             if (zero) {
                 l[0] = nf[0];
@@ -459,7 +473,8 @@ __global__ void __launch_bounds__(tail_threads<T>()) k_tail_levels(const __grid_
                     y0[a] = c[a];
                     z[a] = l[a];
                 }
-                const V v = fma2(gt, z[a], fma2(c0, y0[a], fma2(mt, l[a], fma2(nu, m2[a], mul2(mu, c[a])))));
+                // from the small terms to the large ones
+                const V v = fma2(mu, c[a], fma2(nu, m2[a], fma2(c0, y0[a], fma2(mt_gt.x, l[a], mul2(mt_gt.y, z[a])))));
                 m2[a] = c[a];
                 c[a] = v;
             }
@@ -583,7 +598,7 @@ __global__ void __launch_bounds__(tail_threads<T>()) k_tail_levels(const __grid_
                         const T nu = T(1) - mu, mt = mu * tu;
 #pragma unroll
                         for (int a = 0; a < 2; ++a) {
-                            const V v = fma2(mt, l[a], fma2(nu, prev[a], mul2(mu, c[a])));
+                            const V v = fma2(mu, c[a], fma2(nu, prev[a], mul2(mt, l[a])));
                             prev[a] = c[a];
                             c[a] = v;
                         }
@@ -926,6 +941,8 @@ bool tail_plan(TailParams<T>& p, bool twod, TailLaunch* out) {
         words += 2 * (size_t)L.fld;
         L.f = (int)words;
         words += (size_t)2 * pairs * L.nx * L.ny;
+        L.scaled = (int)words;                   // (even, as every size before it)
+        if (l < p.nl - 1) words += 2 * (size_t)p.s;
         if (words * sizeof(T) > kSmemLimit) return false;
         L.inv_cells = T(1.0 / double(cells));
         L.inv_nq = 1.0f / float(L.nx / 2);

@@ -664,13 +664,13 @@ bool tail_params(const sg_grid* g, int L, int B, TailParams<W>& p, TailLaunch* t
     p.order = order;
     p.s = s;
     p.gsrb = g->opt.smoother == SG_SMOOTH_GSRB ? 1 : 0;
-    p.mut1 = W(r.mut[1]);
+    p.mut[1] = r.mut[1];
     for (int j = 2; j <= s; ++j) {
         p.mu[j] = W(r.mu[j]);
         p.nu[j] = W(r.nu[j]);
-        p.mut[j] = W(r.mut[j]);
+        p.mut[j] = r.mut[j];
         p.c0[j] = W(r.c0[j]);
-        p.gt[j] = W(r.gt[j]);
+        p.gt[j] = r.gt[j];
     }
     for (int i = 0; i < p.nl; ++i) {
         const Level& lv = g->lv[B + i];
@@ -685,7 +685,7 @@ bool tail_params(const sg_grid* g, int L, int B, TailParams<W>& p, TailLaunch* t
         q.hy = g->twod ? W(0) : ih2y<W>(G);
         q.hz = g->twod ? ih2y<W>(G) : ih2z<W>(G);
         q.md = W(-2) * (q.hx + q.hy + q.hz);
-        q.tau = W(g->opt.tau_frac * (2.0 / lambda_max(lv)) * r.tau_over_dtpar);
+        q.tau = g->opt.tau_frac * (2.0 / lambda_max(lv)) * r.tau_over_dtpar;
         q.omega = W(gsrb_omega(g, B + i));
         for (int d = 0; d < 3; ++d) p.per[d] = G.per[d];
         if (g->twod) p.per[2] = G.per[1];

@@ -265,10 +265,12 @@ struct TailLevel {
     int nx, ny, nz;                      // two-dimensional levels: nx x 1 x ny
     int n_pre, n_post;
     T hx, hy, hz, md;                    // 1 / h^2, -2 (hx + hy + hz)
-    T tau, omega, inv_cells;
+    double tau;
+    T omega, inv_cells;
     int split;                           // cut into z slabs over the cluster
     int group;                           // threads that work on it: 0 the whole CTA, 1 four warps, 2 one warp
     int row, fld, buf, f;                // row stride, size of a buffer, offsets of the two buffers and of f
+    int scaled;                          // offset of mu~_j tau, gamma~_j tau (j = 1 .. s)
     float inv_nq, inv_ny, inv_pairs;     // 1 / (nx / 2), 1 / ny (two-dimensional: 1), 1 / (nz / 2)
     short first[17];                     // first plane pair of each CTA (split levels)
 };
@@ -277,7 +279,8 @@ struct TailParams {
     int nl;                              // levels, finest first
     int per[3];
     int order, s, gsrb;
-    T mut1, mu[kTailMaxS + 1], nu[kTailMaxS + 1], mut[kTailMaxS + 1], c0[kTailMaxS + 1], gt[kTailMaxS + 1];
+    T mu[kTailMaxS + 1], nu[kTailMaxS + 1], c0[kTailMaxS + 1];
+    double mut[kTailMaxS + 1], gt[kTailMaxS + 1];
     int remove_mean;                     // every axis periodic: f -= mean(f) below the first level
     const int* sched;                    // coarse solve: s per super-step (device)
     int max_ss;
