@@ -4,6 +4,9 @@
 #pragma once
 #include "sg_internal.cuh"
 
+#include <algorithm>
+#include <cmath>
+
 namespace sg {
 
 namespace {
@@ -208,30 +211,63 @@ __device__ __forceinline__ void store_out(float* dst, float4 v, bool vec, int n)
     }
 }
 
+// The spacing of the FP32 numbers at x.
+inline double spacing_f32(double x) { return x == 0.0 ? 0.0 : std::ldexp(1.0, std::ilogb(x) - 23); }
+
+// FP32 coefficients a of the axes' neighbour sums, near a0, and b = m - 2 (ax + ay + az)
+// of the cell itself (m: an FP32 number) without rounding: an error of b acts on the cell,
+// one of ax on a second difference only.  The sum of the a is taken on the grid on which b
+// is an FP32 number; the axis that the difference moves least takes it.
+inline void sum_exact(double m, const double a0[3], float* a[3], float* b) {
+    const double sum = a0[0] + a0[1] + a0[2];
+    // (1 + 1e-6: also where rounding takes b past a power of two)
+    const double q = 0.5 * std::max(spacing_f32(m), spacing_f32((m - 2.0 * sum) * (1.0 + 1e-6)));
+    const double on_grid = q > 0.0 ? q * std::nearbyint(sum / q) : sum;
+    for (int d = 0; d < 3; ++d) *a[d] = float(a0[d]);
+    int best = -1;
+    double best_v = 0.0, best_r = 0.0;
+    for (int d = 0; d < 3; ++d) {
+        const double v = on_grid - double(*a[(d + 1) % 3]) - double(*a[(d + 2) % 3]);
+        const double r = std::fabs(v - a0[d]) / std::fabs(a0[d]);
+        if (a0[d] == 0.0 || double(float(v)) != v || !(best < 0 || r < best_r)) continue;
+        best = d;
+        best_v = v;
+        best_r = r;
+    }
+    if (best >= 0) *a[best] = float(best_v);
+    *b = float(m - 2.0 * (double(*a[0]) + double(*a[1]) + double(*a[2])));
+}
+
+// The weights of the cell's own values add up without rounding too: b + 2 (ax + ay + az) =
+// mu_j, and 1 - mu_j for Y0.  (All coefficients rounded one by one, a super-step of s = 3 of
+// a smooth 30 x 62 x 46 field in cells of three widths was off by 2.0e-7; by 1.0e-7 so, as
+// stage by stage.)
 inline LeanCoef make_lean_coef(const LevelGeom& g, int order, int s, const FusedCoef& cf) {
     LeanCoef k{};
     const double hx = g.ihx2f, hy = g.ihy2f, hz = g.ihz2f;
     const double tau = cf.tau;
+    double mu[4] = {};
     for (int j = 2; j <= s; ++j) {
         const double mt = cf.mut_tau[j];
-        k.ax[j] = float(mt * hx);
-        k.ay[j] = float(mt * hy);
-        k.az[j] = float(mt * hz);
-        k.b[j] = float(double(cf.mu[j]) - 2.0 * mt * (hx + hy + hz));
+        const double a0[3] = {mt * hx, mt * hy, mt * hz};
+        const double b0 = double(cf.mu[j]) - 2.0 * (a0[0] + a0[1] + a0[2]);
+        const double q = spacing_f32(b0 * (1.0 + 1e-6));
+        mu[j] = q > 0.0 ? q * std::nearbyint(cf.mu[j] / q) : double(cf.mu[j]);
+        float* a[3] = {&k.ax[j], &k.ay[j], &k.az[j]};
+        sum_exact(mu[j], a0, a, &k.b[j]);
     }
-    k.ihx2 = g.ihx2f;
-    k.ihy2 = g.ihy2f;
-    k.ihz2 = g.ihz2f;
-    k.m2s = float(-2.0 * (hx + hy + hz));
+    const double h0[3] = {hx, hy, hz};
+    float* h[3] = {&k.ihx2, &k.ihy2, &k.ihz2};
+    sum_exact(0.0, h0, h, &k.m2s);
     k.m1t = float(double(cf.mut1) * tau);
-    const double c0_2 = order == 2 ? cf.c0[2] : 0.0, gt_2 = order == 2 ? cf.gt[2] : 0.0;
-    k.k2y0 = float(double(cf.nu[2]) + c0_2);
+    const double gt_2 = order == 2 ? cf.gt[2] : 0.0;
+    k.k2y0 = float(1.0 - mu[2]);                    // nu_2 + c0_2
     k.k2z = float(gt_2 * tau);
     k.k2f = float(-double(cf.mut_tau[2]));
     if (s >= 3) {
-        const double c0_3 = order == 2 ? cf.c0[3] : 0.0, gt_3 = order == 2 ? cf.gt[3] : 0.0;
+        const double gt_3 = order == 2 ? cf.gt[3] : 0.0;
         const double nu3 = cf.nu[3];
-        k.k3c = float(nu3 + c0_3);
+        k.k3c = float(1.0 - mu[3]);                 // nu_3 + c0_3
         k.k3l = float(nu3 * double(cf.mut1) * tau + gt_3 * tau);
         k.k3f = float(-double(cf.mut_tau[3]));
     }

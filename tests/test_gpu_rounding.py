@@ -54,3 +54,22 @@ def test_vcycle_in_the_cluster_launch(shape, bc, hi, opts):
         e[precision, fused] = g.potential()
     ref = e["fp64", 0]
     assert _off(e["mixed", 1], ref) < 1.5 * _off(e["mixed", 0], ref)
+
+
+@pytest.mark.parametrize("shape,hi", [((30, 62, 46), (0.6, 1.0, 0.8)), ((56, 40, 72), (1.1, 0.7, 1.3)), ((48, 48, 48), (1.0, 1.0, 1.0))])
+@pytest.mark.parametrize("order", [1, 2])
+@pytest.mark.parametrize("source", [0.0, -30.0])
+def test_fused_superstep(shape, hi, order, source):
+    # s = 3, the fused super-step against the three stage launches
+    sg = _sg()
+    u = _smooth(shape, 5)
+    f = (source * u * (1.0 + 0.1 * np.random.default_rng(7).standard_normal(shape))).astype(np.float32)
+    out = {}
+    for precision, fused, t in (("fp64", 0, torch.float64), ("mixed", 0, torch.float32), ("mixed", 1, torch.float32)):
+        g = sg.Grid(shape, (0.0, 0.0, 0.0), hi, (0, 0, 0), precision=precision)
+        g.set_options(fused=fused)
+        o = torch.empty(shape, dtype=t, device="cuda")
+        g.op_superstep(0, order, 3, 0.9, torch.tensor(u, dtype=t, device="cuda"), torch.tensor(f, dtype=t, device="cuda"), o)
+        out[precision, fused] = o.double().cpu().numpy()
+    ref = out["fp64", 0]
+    assert _off(out["mixed", 1], ref) < 1.5 * _off(out["mixed", 0], ref)
