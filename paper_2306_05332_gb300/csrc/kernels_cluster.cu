@@ -830,7 +830,9 @@ __global__ void __launch_bounds__(tail_threads<T>()) k_tail_levels(const __grid_
         }
     }
     cl.sync();                                   // peers may still read or write this CTA's memory until here
-    if (!waits_ok) {                             // a bounded wait gave up: the solve reports a non-finite residual
+    // a bounded wait gave up: the solve reports a non-finite residual (from the update's
+    // norm; a resident solve from the residual of phi that loop_confirm reads)
+    if (!waits_ok) {
         atomicAdd(&g_tail_wait_timeouts, 1u);
         if (stay) p.phi[0] = __longlong_as_double(0x7ff8000000000000ll);
         else p.u_out[0] = T(__int_as_float(0x7fc00000));

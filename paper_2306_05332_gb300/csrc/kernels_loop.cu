@@ -16,20 +16,6 @@ namespace sg {
 
 namespace {
 
-__device__ __forceinline__ bool loop_met(const DeviceLoop& d, double rel, double maxabs) {
-    return d.mtol > 0.0 ? maxabs <= d.mtol : rel <= d.tol;
-}
-
-__device__ __forceinline__ double loop_rel(const DeviceLoop& d, const Reduced& r) {
-    return sqrt(r.sumsq / d.nn) / d.rden;
-}
-
-__device__ __forceinline__ void loop_record(DeviceLoop& d, double rel, double maxabs) {
-    if (d.m < kLoopHistory) d.history[d.m] = rel;
-    d.rel = rel;
-    d.maxabs = maxabs;
-}
-
 // After a cycle: fold the residual's block partials (a launch of its own cost 2.5 us a
 // cycle), count the cycle and decide whether the inner loop runs another.
 __global__ void __launch_bounds__(kRedThreads)
@@ -49,26 +35,14 @@ k_loop_step(DeviceLoop* dl, const Partial* partials, int nb, Reduced* red, const
     cudaGraphSetConditional(inner, go ? 1u : 0u);
 }
 
-// After the inner loop (mixed precision: the true FP64 residual is in red):
-// confirm, or resume the cycles.
-// (nb > 0: the residual's partials)
+// After the inner loop: confirm, or resume the cycles (nb > 0: mixed precision, the
+// partials of the true FP64 residual).
 __global__ void __launch_bounds__(kRedThreads)
 k_loop_confirm(DeviceLoop* dl, const Partial* partials, int nb, Reduced* red, cudaGraphConditionalHandle outer,
                cudaGraphConditionalHandle inner, int has_inner) {
     if (nb > 0) fold_partials(partials, nb, red);
     if (threadIdx.x != 0) return;
-    DeviceLoop& d = *dl;
-    unsigned go = 0;
-    d.confirms += 1;
-    if (d.pending) {
-        d.pending = 0;
-        const double rel = loop_rel(d, *red), maxabs = red->maxabs;
-        loop_record(d, rel, maxabs);
-        if (!isfinite(rel)) d.status = kLoopNonFinite;
-        else if (loop_met(d, rel, maxabs)) d.status = kLoopDone;
-        else if (d.m >= d.limit) d.status = kLoopNotConverged;
-        else go = 1;
-    }
+    const unsigned go = loop_confirm(*dl, *red) ? 1u : 0u;
     if (has_inner) cudaGraphSetConditional(inner, go);
     cudaGraphSetConditional(outer, go);
 }

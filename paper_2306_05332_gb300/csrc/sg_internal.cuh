@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <cstdint>
 #include <cstddef>
 
@@ -176,12 +177,18 @@ cudaError_t launch_loop_step(DeviceLoop* d, const Partial* partials, int nb, Red
 cudaError_t launch_loop_confirm(DeviceLoop* d, const Partial* partials, int nb, Reduced* red,
                                 cudaGraphConditionalHandle outer, cudaGraphConditionalHandle inner, bool has_inner,
                                 cudaStream_t st);
+__host__ __device__ __forceinline__ bool loop_met(const LoopState& d, double rel, double maxabs) {
+    return d.mtol > 0.0 ? maxabs <= d.mtol : rel <= d.tol;
+}
+__host__ __device__ __forceinline__ double loop_rel(const LoopState& d, const Reduced& r) {
+    return sqrt(r.sumsq / d.nn) / d.rden;
+}
 // The decision after a cycle with relative residual rel and largest residual maxabs, on
 // the counters of d: true to run another.  *record: the residual goes into the history.
-__device__ __forceinline__ bool loop_decide(LoopState& d, double rel, double maxabs, bool* record) {
+__host__ __device__ __forceinline__ bool loop_decide(LoopState& d, double rel, double maxabs, bool* record) {
     d.m += 1;
     const bool finite = isfinite(rel);
-    const bool met = d.mtol > 0.0 ? maxabs <= d.mtol : rel <= d.tol;
+    const bool met = loop_met(d, rel, maxabs);
     *record = true;
     if (!d.fixed && finite && met && d.confirm) {
         d.pending = 1;                      // the true residual decides (k_loop_confirm)
@@ -193,6 +200,25 @@ __device__ __forceinline__ bool loop_decide(LoopState& d, double rel, double max
     if (!finite) d.status = kLoopNonFinite;
     else if (!d.fixed && met) d.status = kLoopDone;
     else if (d.m >= d.limit) d.status = d.fixed ? kLoopDone : kLoopNotConverged;
+    else return true;
+    return false;
+}
+// The decision after the inner loop, red: the residual f - A phi (mixed precision), else that
+// of the last cycle; true to resume the cycles.  A residual that is not finite ends the
+// solve as such also where nothing waits for the confirmation (a fixed cycle count, the
+// cycle cap): a launch that gave up a wait leaves its NaN in phi after its last decision.
+__host__ __device__ __forceinline__ bool loop_confirm(DeviceLoop& d, const Reduced& red) {
+    d.confirms += 1;
+    const double rel = loop_rel(d, red);
+    const bool finite = isfinite(rel);
+    if (!d.pending && finite) return false;
+    d.pending = 0;
+    if (d.m < kLoopHistory) d.history[d.m] = rel;
+    d.rel = rel;
+    d.maxabs = red.maxabs;
+    if (!finite) d.status = kLoopNonFinite;
+    else if (loop_met(d, rel, red.maxabs)) d.status = kLoopDone;
+    else if (d.m >= d.limit) d.status = kLoopNotConverged;
     else return true;
     return false;
 }

@@ -1,0 +1,82 @@
+"""What the host does with failures and options, without a GPU: ``sg_host.cu`` linked with
+launchers and a CUDA runtime that run nothing (``fake_device.cpp``), through the package's
+own binding.
+"""
+
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+import paper_2306_05332_gb300 as sg
+from paper_2306_05332_gb300 import build as B
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+RUNNING, DONE, NOT_CONVERGED = 0, 1, 2           # DeviceLoop::status
+
+
+@pytest.fixture(scope="module")
+def fake_lib(tmp_path_factory):
+    if shutil.which("nvcc") is None and not os.path.exists("/usr/local/cuda/bin/nvcc"):
+        pytest.skip("nvcc not found")
+    d = tmp_path_factory.mktemp("fake")
+    include = ["-I", os.path.join(B.ROOT, "include"), "-I", B.CSRC]
+    host, fake, so = (str(d / n) for n in ("sg_host.o", "fake_device.o", "libsg_fake.so"))
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(B.nvcc()))), "include")
+    for cmd in ([B.nvcc(), *B.ARCH, "-O1", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr", *include,
+                 "-c", os.path.join(B.CSRC, "sg_host.cu"), "-o", host],
+                ["g++", "-O1", "-std=c++17", "-fPIC", "-w", *include, "-I", cuda,
+                 "-c", os.path.join(HERE, "fake_device.cpp"), "-o", fake],
+                ["g++", "-shared", "-Wl,-Bsymbolic", "-Wl,-z,defs", "-o", so, host, fake, "-lpthread"]):
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        assert r.returncode == 0, r.stderr
+    L = ctypes.CDLL(so)
+    for name, (args, res) in sg._SIGS.items():
+        getattr(L, name).argtypes, getattr(L, name).restype = args, res
+    L.fake_norm.argtypes = [ctypes.c_double]
+    L.fake_loop.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_double]
+    return L
+
+
+@pytest.fixture
+def fake(fake_lib, monkeypatch):
+    monkeypatch.setattr(sg, "_LIB", fake_lib)
+    monkeypatch.setattr(sg, "_torch", lambda: None)
+    fake_lib.fake_reset()
+    return fake_lib
+
+
+def _grid(shape, precision="mixed", **opts):
+    g = sg.Grid(shape, precision=precision)
+    if opts:
+        g.set_options(**opts)
+    g.set_density(np.ones(shape), 1.0)
+    return g
+
+
+@pytest.mark.parametrize("opts,tol,status", [(dict(fixed_cycles=3), 0.0, DONE),
+                                             (dict(max_cycles=1), 1e-9, NOT_CONVERGED)])
+def test_nan_left_after_the_last_decision_is_reported(fake, opts, tol, status):
+    # a launch that gave up a wait: the loop has ended with a finite residual, the
+    # potential holds a NaN, so the residual of the potential is one
+    g = _grid((32, 32, 32), **opts)
+    fake.fake_loop(status, 0, float("nan"))
+    fake.fake_waits(0, 1)
+    info = g.solve(tol=tol, check=False)
+    assert info["status"] == "SG_ERR_NONFINITE"
+    assert np.isnan(info["rel_residual"])
+    assert b"gave up a bounded wait" in fake.sg_last_error()
+
+
+@pytest.mark.parametrize("status,pending,sumsq,want", [(DONE, 0, 1.0, "SG_OK"), (NOT_CONVERGED, 0, 1.0, "SG_ERR_NOT_CONVERGED"),
+                                                       (RUNNING, 1, 0.0, "SG_OK"), (RUNNING, 1, float("inf"), "SG_ERR_NONFINITE")])
+def test_decision_after_the_inner_loop(fake, status, pending, sumsq, want):
+    g = _grid((32, 32, 32), fixed_cycles=0 if pending else 3)
+    fake.fake_loop(status, pending, sumsq)
+    info = g.solve(tol=1e-9, check=False)
+    assert info["status"] == want
+    if not pending:
+        assert info["rel_residual"] == 0.5            # the loop's own, not the confirmation's
