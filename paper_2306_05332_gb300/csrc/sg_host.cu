@@ -1101,6 +1101,14 @@ sg_status solve_begin(sg_grid* g, SolveState& S, double tol, int L, double* phi,
     return solve_begin_finish(g, S, have_guess);
 }
 
+// (both precisions: FP64 solves run the cluster launch and its bounded waits too)
+sg_status fail_nonfinite() {
+    const unsigned waits = lean_wait_failures() + tail_wait_failures();
+    return fail(SG_ERR_NONFINITE, waits ? "residual norm is not finite: " + std::to_string(waits) +
+                                              " launch(es) gave up a bounded wait"
+                                        : std::string("residual norm is not finite"));
+}
+
 // Record the residual now in host_red[0]; decide whether the solve is over.
 // Mixed precision carries the FP64 residual by recurrence between cycles; when
 // it reaches the tolerance, the true FP64 residual f - A phi is computed once to
@@ -1123,10 +1131,7 @@ sg_status solve_check(sg_grid* g, SolveState& S) {
     S.info.rel_residual = rel;
     S.info.max_residual = g->host_red[0].maxabs;
     if (!std::isfinite(rel)) {
-        const unsigned waits = g->precision == SG_MIXED ? lean_wait_failures() + tail_wait_failures() : 0u;
-        S.status = fail(SG_ERR_NONFINITE, waits ? "residual norm is not finite: " + std::to_string(waits) +
-                                                      " launch(es) gave up a bounded wait"
-                                                : std::string("residual norm is not finite"));
+        S.status = fail_nonfinite();
         S.done = true;
     } else if (g->opt.fixed_cycles == 0 && met(rel, g->host_red[0].maxabs)) {
         S.done = true;
@@ -1329,10 +1334,7 @@ void read_device_loop(sg_grid* g, SolveState& S, const DeviceLoop& d, long long 
     S.su += (long long)(d.m - m0) * stage_updates_per_cycle(g, S.L) + d.coarse_stage_cells;
     g->launches += 1 + (long long)(d.m - m0) * per_cycle + (long long)d.confirms * per_confirm;
     if (d.status == kLoopNonFinite) {
-        const unsigned waits = g->precision == SG_MIXED ? lean_wait_failures() + tail_wait_failures() : 0u;
-        S.status = fail(SG_ERR_NONFINITE, waits ? "residual norm is not finite: " + std::to_string(waits) +
-                                                      " launch(es) gave up a bounded wait"
-                                                : std::string("residual norm is not finite"));
+        S.status = fail_nonfinite();
     } else if (d.status == kLoopNotConverged) {
         S.status = fail(SG_ERR_NOT_CONVERGED, "max_cycles reached above the tolerance");
     }

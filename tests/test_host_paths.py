@@ -15,7 +15,7 @@ import paper_2306_05332_gb300 as sg
 from paper_2306_05332_gb300 import build as B
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-RUNNING, DONE, NOT_CONVERGED = 0, 1, 2           # DeviceLoop::status
+RUNNING, DONE, NOT_CONVERGED, NON_FINITE = 0, 1, 2, 3           # DeviceLoop::status
 
 
 @pytest.fixture(scope="module")
@@ -80,3 +80,15 @@ def test_decision_after_the_inner_loop(fake, status, pending, sumsq, want):
     assert info["status"] == want
     if not pending:
         assert info["rel_residual"] == 0.5            # the loop's own, not the confirmation's
+
+
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+def test_waits_are_named_in_both_precisions(fake, precision):
+    g = _grid((32, 32, 32), precision)
+    fake.fake_waits(0, 1)
+    fake.fake_loop(NON_FINITE, 0, float("nan"))
+    assert g.solve(tol=1e-9, check=False)["status"] == "SG_ERR_NONFINITE"        # in a cycle
+    assert b"gave up a bounded wait" in fake.sg_last_error()
+    fake.fake_norm(float("nan"))
+    assert g.solve(tol=1e-9, check=False)["status"] == "SG_ERR_NONFINITE"        # at the first residual
+    assert b"gave up a bounded wait" in fake.sg_last_error()
