@@ -257,7 +257,7 @@ __device__ __forceinline__ bool wait_phase(unsigned bar, unsigned parity) {
     }
     return false;
 }
-// Waits that gave up since the library was loaded.
+// Launches with a wait that gave up since the library was loaded.
 __device__ unsigned int g_tail_wait_timeouts = 0;
 
 template <typename T, bool TWOD>
@@ -286,8 +286,12 @@ __global__ void __launch_bounds__(tail_threads<T>()) k_tail_levels(const __grid_
     const int tid = threadIdx.x, lane = tid & 31;
     int rslot = 0;
     unsigned xn = 0;                             // exchanges so far, the same count in every CTA
+    // After a wait that gave up the thread neither arms a barrier (a phase that is not
+    // complete must not be armed again) nor sends; its neighbours give up in their turn.
     bool waits_ok = true;
+    __shared__ int gave_up;                      // on CTA 0: some thread of the cluster did
     if (tid == 0) {
+        gave_up = 0;
         for (int b = 0; b < 2; ++b)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((unsigned)__cvta_generic_to_shared(&xbar[b]))
                          : "memory");
@@ -360,7 +364,7 @@ __global__ void __launch_bounds__(tail_threads<T>()) k_tail_levels(const __grid_
     // sends those cells, so data of a neighbour's next exchange cannot overtake a read.
     auto publish = [&](const H& h, auto split, int off, const V (&c)[2]) {
         if constexpr (decltype(split)::value) {
-            if (tid == 0)
+            if (tid == 0 && waits_ok)
                 asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(
                                  (unsigned)__cvta_generic_to_shared(&xbar[xn & 1])),
                              "r"(h.bytes)
@@ -371,8 +375,8 @@ __global__ void __launch_bounds__(tail_threads<T>()) k_tail_levels(const __grid_
             st(y, c[0]);
             st(y + h.plane, c[1]);
             if constexpr (decltype(split)::value) {
-                if (h.far_lo) st_far(h.far_lo + off * (int)sizeof(T), c[0], h.bar_lo + 8 * (xn & 1));
-                if (h.far_hi) st_far(h.far_hi + off * (int)sizeof(T), c[1], h.bar_hi + 8 * (xn & 1));
+                if (h.far_lo && waits_ok) st_far(h.far_lo + off * (int)sizeof(T), c[0], h.bar_lo + 8 * (xn & 1));
+                if (h.far_hi && waits_ok) st_far(h.far_hi + off * (int)sizeof(T), c[1], h.bar_hi + 8 * (xn & 1));
             }
         }
         group_sync(h.group);
@@ -829,10 +833,14 @@ __global__ void __launch_bounds__(tail_threads<T>()) k_tail_levels(const __grid_
             else if (p.ss_done) *p.ss_done = done;
         }
     }
+    if (!waits_ok) {                             // copies on their way land (microseconds) before a CTA ends
+        *cl.map_shared_rank(&gave_up, 0) = 1;
+        for (int i = 0; i < 1000; ++i) __nanosleep(1000);
+    }
     cl.sync();                                   // peers may still read or write this CTA's memory until here
     // a bounded wait gave up: the solve reports a non-finite residual (from the update's
     // norm; a resident solve from the residual of phi that loop_confirm reads)
-    if (!waits_ok) {
+    if (rank == 0 && tid == 0 && gave_up) {
         atomicAdd(&g_tail_wait_timeouts, 1u);
         if (stay) p.phi[0] = __longlong_as_double(0x7ff8000000000000ll);
         else p.u_out[0] = T(__int_as_float(0x7fc00000));

@@ -329,7 +329,7 @@ struct TailLaunch {
     size_t bytes;
 };
 cudaError_t tail_configure();
-// Bounded waits of this launch that gave up since the library was loaded; each wrote a NaN into its output.
+// Launches of it with a bounded wait that gave up since the library was loaded; each wrote a NaN into its output.
 unsigned tail_wait_failures();
 // Fills the layout of p.lv (sizes and nl set) and the launch shape; false where
 // the levels (and, when p.loop is set, phi and r of the first one) do not fit one
