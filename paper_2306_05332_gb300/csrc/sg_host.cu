@@ -1917,20 +1917,23 @@ sg_status sg_solve_batch(sg_grid* const* grids, int n, double tol, sg_solve_info
     if (par.empty()) return first;
     const size_t P = par.size();
     std::vector<SolveState> S(P);
+    // a start that fails ends the batch with no grid's work in flight and every guess kept
+    auto abandon = [&](sg_status st) {
+        for (int i : par) cudaStreamSynchronize(grids[i]->st);
+        return st;
+    };
     for (size_t k = 0; k < P; ++k) {
         sg_grid* g = grids[par[k]];
         const sg_status st = solve_begin_enqueue(g, S[k], tol, g->max_levels, g->phi, g->f, g->have_faces, g->guess_set);
-        if (st != SG_OK) {                      // the starts before it are left complete
-            for (size_t q = 0; q <= k; ++q) cudaStreamSynchronize(grids[par[q]]->st);
-            return st;
-        }
+        if (st != SG_OK) return abandon(st);
     }
     for (size_t k = 0; k < P; ++k) {
         sg_grid* g = grids[par[k]];
-        SG_TRY(solve_begin_finish(g, S[k], g->guess_set));
-        g->guess_set = false;
-        SG_TRY(solve_check(g, S[k]));
+        sg_status st = solve_begin_finish(g, S[k], g->guess_set);
+        if (st == SG_OK) st = solve_check(g, S[k]);
+        if (st != SG_OK) return abandon(st);
     }
+    for (int i : par) grids[i]->guess_set = false;
     // the batch graph, kept while the same grids (by serial number) with the
     // same keys come back
     std::vector<uint64_t> key;

@@ -161,6 +161,7 @@ cudaError_t launch_gsrb(const LevelGeom& g, int, double, T*, const T*, cudaStrea
 }
 template <typename TI, typename TO>
 cudaError_t launch_residual(const LevelGeom&, const TI*, const TI*, TO*, Partial*, int* nb, cudaStream_t st, TI*) {
+    if (!g_capturing) log("residual", {});
     if (nb) *nb = 1;
     return busy(st);
 }
@@ -189,6 +190,7 @@ cudaError_t launch_finalize(const Partial*, int, Reduced* out, cudaStream_t st) 
 }
 cudaError_t launch_residual_exact(const LevelGeom&, const double*, const double*, float*, double*, Partial*, unsigned*,
                                   int* nb, int* nk, cudaStream_t st) {
+    if (!g_capturing) log("residual", {});
     if (nb) *nb = 1;
     if (nk) *nk = 2;
     return busy(st);

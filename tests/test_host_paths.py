@@ -57,6 +57,16 @@ def _grid(shape, precision="mixed", **opts):
     return g
 
 
+def _log(fake, what):
+    out = []
+    for i in range(fake.fake_log_size()):
+        name, v = ctypes.create_string_buffer(16), (ctypes.c_double * 8)()
+        fake.fake_log_entry(i, name, v)
+        if name.value.decode() == what:
+            out.append(list(v))
+    return out
+
+
 @pytest.mark.parametrize("opts,tol,status", [(dict(fixed_cycles=3), 0.0, DONE),
                                              (dict(max_cycles=1), 1e-9, NOT_CONVERGED)])
 def test_nan_left_after_the_last_decision_is_reported(fake, opts, tol, status):
@@ -92,3 +102,22 @@ def test_waits_are_named_in_both_precisions(fake, precision):
     fake.fake_norm(float("nan"))
     assert g.solve(tol=1e-9, check=False)["status"] == "SG_ERR_NONFINITE"        # at the first residual
     assert b"gave up a bounded wait" in fake.sg_last_error()
+
+
+@pytest.mark.parametrize("nth", [1, 2, 3])
+def test_batch_whose_start_fails_leaves_nothing_in_flight_and_keeps_the_guesses(fake, nth):
+    # (the first allocations of a batch are its grids' coarse schedules)
+    grids = [_grid((16, 16, 16)), _grid((32, 32, 32)), _grid((24, 24, 24))]
+    for g in grids:
+        g.set_guess(np.zeros(g.shape))
+    fake.fake_reset()
+    fake.fake_fail_alloc(nth)
+    with pytest.raises(sg.SGError):
+        sg.solve_batch(grids, tol=1e-9)
+    assert fake.fake_busy() == 0
+    fake.fake_reset()
+    sg.solve_batch(grids, tol=1e-9)
+    assert len(_log(fake, "residual")) == 3         # the residual of each guess
+    fake.fake_reset()
+    sg.solve_batch(grids, tol=1e-9)
+    assert len(_log(fake, "residual")) == 0         # a guess is taken once
