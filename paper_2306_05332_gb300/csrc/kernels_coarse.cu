@@ -11,6 +11,7 @@
 // Boundaries: homogeneous Dirichlet (Eq. error_ghost) or periodic.
 #include "sg_internal.cuh"
 
+#include <algorithm>
 #include <cstdint>
 #include <type_traits>
 
@@ -58,7 +59,10 @@ __device__ T block_sum(T v, T* scratch) {
 // n <= kSmemLimit / (4 sizeof(float)) < kMaxCells * kCoarseThreads.
 constexpr int kMaxCells = 16;
 
-template <typename T, int MAXC>
+// LONG: an extent above 1024.  The packed coordinates then take as many bits as the
+// extents need (17 at most, n < 2^14) instead of ten each; the variable shifts cost
+// registers (MAXC = 16: spills), so other levels keep the fixed fields.
+template <typename T, int MAXC, bool LONG>
 __global__ void __launch_bounds__(kCoarseThreads) k_coarse_solve(const CoarseParams p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ T red[33];
@@ -71,14 +75,16 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_solve(const CoarsePar
     int per[3] = {p.g.per[0], p.g.per[1], p.g.per[2]};
 
     // this thread's cells t = tid + m * blockDim, coordinates packed once
+    const int bx = LONG ? 32 - __clz(nx - 1) : 10, by = LONG ? 32 - __clz(ny - 1) : 10, bxy = bx + by;
+    const int mx = (1 << bx) - 1, my = (1 << by) - 1;
     int cell[MAXC];
 #pragma unroll
     for (int m = 0; m < MAXC; ++m) {
         const int t = threadIdx.x + m * blockDim.x;
-        cell[m] = t < n ? ((t % nx) | (((t / nx) % ny) << 10) | ((t / (nx * ny)) << 20)) : -1;
+        cell[m] = t < n ? ((t % nx) | (((t / nx) % ny) << bx) | ((t / (nx * ny)) << bxy)) : -1;
     }
     auto lap = [&](const T* y, int c) {
-        return lap_smem(y, nx, ny, nz, per, ihx2, ihy2, ihz2, c & 1023, (c >> 10) & 1023, c >> 20);
+        return lap_smem(y, nx, ny, nz, per, ihx2, ihy2, ihz2, c & mx, (c >> bx) & my, c >> bxy);
     };
 
     T local = T(0);
@@ -381,7 +387,7 @@ size_t coarse_smem_bytes(long long n) {
 
 template <typename T>
 bool coarse_fits(long long n) {
-    // shared-memory capacity, the per-thread cell table, and 10-bit packed coordinates
+    // shared-memory capacity and the per-thread cell table
     return coarse_smem_bytes<T>(n) <= kSmemLimit && n <= (long long)kMaxCells * kCoarseThreads;
 }
 
@@ -406,28 +412,33 @@ cudaError_t launch_coarse_solve(const CoarseParams& p, cudaStream_t st) {
         k_coarse_small<T><<<1, threads, small, st>>>(p);
         return cudaGetLastError();
     }
-    if (n <= 4LL * kCoarseThreads) k_coarse_solve<T, 4><<<1, threads, bytes, st>>>(p);
-    else k_coarse_solve<T, kMaxCells><<<1, threads, bytes, st>>>(p);
+    auto run = [&](auto is_long) {
+        constexpr bool LONG = decltype(is_long)::value;
+        if (n <= 4LL * kCoarseThreads) k_coarse_solve<T, 4, LONG><<<1, threads, bytes, st>>>(p);
+        else k_coarse_solve<T, kMaxCells, LONG><<<1, threads, bytes, st>>>(p);
+    };
+    if (std::max({p.g.nx, p.g.ny, p.g.nz}) > 1024) run(std::true_type{});
+    else run(std::false_type{});
     return cudaGetLastError();
 }
 
 cudaError_t coarse_configure() {
-    cudaError_t e;
-    if ((e = cudaFuncSetAttribute(k_coarse_strips, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)kSmemLimit)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_coarse_small<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)kSmemLimit)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_coarse_small<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)kSmemLimit)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_coarse_solve<float, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)kSmemLimit)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_coarse_solve<float, kMaxCells>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit)) != cudaSuccess)
-        return e;
-    if ((e = cudaFuncSetAttribute(k_coarse_solve<double, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)kSmemLimit)) != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_coarse_solve<double, kMaxCells>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)kSmemLimit);
+    cudaError_t e = cudaSuccess;
+    auto whole = [&](auto kernel) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
+    };
+    whole(k_coarse_strips);
+    whole(k_coarse_small<float>);
+    whole(k_coarse_small<double>);
+    whole(k_coarse_solve<float, 4, false>);
+    whole(k_coarse_solve<float, 4, true>);
+    whole(k_coarse_solve<float, kMaxCells, false>);
+    whole(k_coarse_solve<float, kMaxCells, true>);
+    whole(k_coarse_solve<double, 4, false>);
+    whole(k_coarse_solve<double, 4, true>);
+    whole(k_coarse_solve<double, kMaxCells, false>);
+    whole(k_coarse_solve<double, kMaxCells, true>);
+    return e;
 }
 
 template size_t coarse_smem_bytes<float>(long long);
