@@ -102,9 +102,9 @@ __device__ __forceinline__ V neg2(V v) {
 // Plane pairs of a split level: rank r owns pairs [first(r), first(r + 1)).
 __host__ __device__ __forceinline__ int first_pair(int r, int np, int nc) { return r * np / nc; }
 
-// a / n with inv = 1 / n in FP32: (a + 1/2) / n is at least 1 / (2 n) away from an
-// integer, far more than the rounding of the product for the sizes of these levels
-// (a < 2^15, n < 2^11).
+// a / n with inv = 1 / n in FP32, for a + 1/2 < 2^22: (a + 1/2) / n is at least 1 / (2 n)
+// away from an integer, and inv and the product together are off by less than 2^-23 of it.
+// The largest a here is nc plane pairs less one, below 16 x 2^15 for rows of 2^16 cells.
 __host__ __device__ __forceinline__ int quick_div(int a, float inv) { return int((float(a) + 0.5f) * inv); }
 
 // The CTA that owns plane pair p.
