@@ -597,7 +597,9 @@ sg_status coarse_solve(sg_grid* g, int l, const W* rhs, W* u, int* d_done) {
 
 // One fused super-step (FP32, homogeneous or periodic ghosts): out = Y_s(y0),
 // y0 == nullptr meaning Y0 = 0.  by_options: the kernel that tile_rows and staging ask
-// for, otherwise the one with a column per thread (the same bits).
+// for, otherwise the one with a column per thread (the same bits).  They are heeded for
+// first super-steps and on levels of kFusedMinCells; on smaller levels the other
+// super-steps would be slower by that kernel than by stages.
 sg_status superstep_fused(sg_grid* g, int l, int order, int s, double tau_frac, const float* y0,
                           const float* rhs, float* out, bool by_options) {
     const Level& L = g->lv[l];
@@ -775,7 +777,7 @@ sg_status vcycle(sg_grid* g, int L, W* u0, const W* rhs0, bool faces, bool zero0
                     const bool z = zero_start && c == 0;
                     float* out = z ? cur[l] : alt[l];
                     SG_TRY(superstep_fused(g, l, g->opt.rkl_order, g->opt.s_smooth, g->opt.tau_frac,
-                                           z ? nullptr : cur[l], R(l), out, g->lv[l].n >= kFusedMinCells));
+                                           z ? nullptr : cur[l], R(l), out, z || g->lv[l].n >= kFusedMinCells));
                     if (!z) std::swap(cur[l], alt[l]);
                 }
                 if (zero_start && count == 0) SG_CK(cudaMemsetAsync(cur[l], 0, g->lv[l].n * sizeof(W), g->st));
@@ -783,7 +785,7 @@ sg_status vcycle(sg_grid* g, int L, W* u0, const W* rhs0, bool faces, bool zero0
             }
             if (zero_start && count > 0 && use_fused_zero(g, fc, l)) {
                 SG_TRY(superstep_fused(g, l, g->opt.rkl_order, g->opt.s_smooth, g->opt.tau_frac, nullptr, R(l),
-                                       cur[l], false));
+                                       cur[l], true));
                 return relax<W>(g, l, count - 1, fc, cur[l], R(l));
             }
         }

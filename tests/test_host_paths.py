@@ -121,3 +121,13 @@ def test_batch_whose_start_fails_leaves_nothing_in_flight_and_keeps_the_guesses(
     fake.fake_reset()
     sg.solve_batch(grids, tol=1e-9)
     assert len(_log(fake, "residual")) == 0         # a guess is taken once
+
+
+@pytest.mark.parametrize("s_smooth", [2, 3])
+@pytest.mark.parametrize("opts,want", [(dict(), (0, 0)), (dict(tile_rows=14), (14, 0)), (dict(tile_rows=16, staging="tma"), (16, 1))])
+def test_first_supersteps_heed_tile_rows_and_staging(fake, s_smooth, opts, want):
+    g = _grid((64, 64, 64), fixed_cycles=1, use_graph=0, s_smooth=s_smooth, **opts)
+    g.solve(tol=0.0, check=False)
+    first = [e for e in _log(fake, "superstep") if e[3] == 1.0]
+    assert len(first) == 1 and first[0][0] == 64 ** 3
+    assert (first[0][4], first[0][5]) == want
