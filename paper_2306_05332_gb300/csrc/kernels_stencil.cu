@@ -410,19 +410,19 @@ void launch_stage64_v(int order, bool first, bool faces, bool uniform, dim3 grid
     else go(Two{}, std::false_type{}, std::true_type{});
 }
 
-// c.tau is 1 and c.mut1, c.gt carry the factor tau (superstep): Z0 = L Y0 - f.
+// Z0 = L Y0 - f without the factor tau: mu~_1 and gamma~_j take it.
 cudaError_t launch_stage64(const LevelGeom& g, int order, bool first, const StageCoef& c, const double* ym1,
                            const double* ym2, const double* y0, const double* z0, const double* rhs, double* out,
                            double* z0_out, cudaStream_t st) {
     Stage64 cf{};
-    cf.m1t = c.mut1;
+    cf.m1t = c.mut1 * c.tau;
     cf.mu = c.mu;
     const double w = first ? 1.0 : c.mut_tau;
     cf.ax = w * g.ihx2;
     cf.ay = w * g.ihy2;
     cf.az = w * g.ihz2;
     cf.kf = -c.mut_tau;
-    cf.kz = c.gt;
+    cf.kz = c.gt * c.tau;
     cf.k0 = c.c0;
     cf.km = c.nu;
     if (order == 2 && !first && ym2 == y0) cf.k0 = c.c0 + c.nu;

@@ -458,11 +458,9 @@ sg_status superstep(sg_grid* g, int l, int order, int s, double tau_frac, bool f
     const double tau = tau_frac * dtpar * r.tau_over_dtpar;
     W* t[3] = {(W*)L.t[0], (W*)L.t[1], (W*)L.t[2]};
     W* z0 = (W*)L.z0;
-    // FP64 stages keep Z0 = L Y0 - f without the factor tau (kernels_stencil.cu)
-    const bool bare = std::is_same<W, double>::value;
     StageCoef c{};
-    c.tau = bare ? 1.0 : tau;
-    c.mut1 = bare ? r.mut[1] * tau : r.mut[1];
+    c.tau = tau;
+    c.mut1 = r.mut[1];
     W* out1 = t[0];
     const int cls = l == 0 ? K_STAGE0 : K_STAGE_C;
     const double nb = double(L.n) * sizeof(W);
@@ -478,11 +476,12 @@ sg_status superstep(sg_grid* g, int l, int order, int s, double tau_frac, bool f
     }
     for (int j = 2; j <= s; ++j) {
         StageCoef cj{};
+        cj.tau = tau;
         cj.mu = r.mu[j];
         cj.nu = r.nu[j];
         cj.mut_tau = r.mut[j] * tau;
         cj.c0 = r.c0[j];
-        cj.gt = bare ? r.gt[j] * tau : r.gt[j];
+        cj.gt = r.gt[j];
         const W* ym1 = (j - 1 == 0) ? u : t[(j - 2) % 3];
         const W* ym2 = (j - 2 == 0) ? u : t[(j - 3) % 3];
         W* out = (j == s) ? u : t[(j - 1) % 3];

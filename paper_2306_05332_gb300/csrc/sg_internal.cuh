@@ -42,8 +42,9 @@ template <> __host__ __device__ __forceinline__ double ih2z<double>(const LevelG
 //   first stage : z = tau (L Y0 - f);  Y1 = Y0 + mut1 * z;   (RKL2 stores z as Z0)
 //   later stages: Yj = mu Y_{j-1} + nu Y_{j-2} + mut_tau (L Y_{j-1} - f)
 //                      [RKL2: + c0 Y0 + gt Z0]
+// (FP64 stages store Z0 without its factor tau and apply it with gt.)
 struct StageCoef {
-    double tau;       // first stage only
+    double tau;
     double mut1;      // first stage only: mu~_1
     double mu, nu;
     double mut_tau;   // mu~_j * tau

@@ -131,3 +131,22 @@ def test_first_supersteps_heed_tile_rows_and_staging(fake, s_smooth, opts, want)
     first = [e for e in _log(fake, "superstep") if e[3] == 1.0]
     assert len(first) == 1 and first[0][0] == 64 ** 3
     assert (first[0][4], first[0][5]) == want
+
+
+@pytest.mark.parametrize("order", [1, 2])
+def test_stage_coefficients_mean_the_same_in_both_precisions(fake, order):
+    stages = {}
+    for precision in ("fp64", "mixed"):
+        g = _grid((8, 8, 8), precision, fixed_cycles=1, use_graph=0, fused=0, rkl_order=order, s_smooth=3, n_pre=1, n_post=0)
+        g.solve(tol=0.0, check=False)
+        # cells, order, first, tau, mu~_1, mu~_j tau, gamma~_j
+        stages[precision] = [e[:7] for e in _log(fake, "stage") if e[0] == 512]
+        fake.fake_reset()
+    assert len(stages["fp64"]) == 3 and stages["fp64"] == stages["mixed"]
+    mut = (ctypes.c_double * 4)()
+    ratio = ctypes.c_double()
+    fake.sg_plan_stage_coefficients(order, 3, None, None, mut, None, ctypes.byref(ratio))
+    tau = 2.0 / (12.0 * 64.0) * ratio.value
+    assert [e[3] for e in stages["fp64"]] == pytest.approx([tau] * 3, rel=1e-14)
+    assert stages["fp64"][0][4] == mut[1]
+    assert [e[5] for e in stages["fp64"][1:]] == pytest.approx([mut[2] * tau, mut[3] * tau], rel=1e-14)
