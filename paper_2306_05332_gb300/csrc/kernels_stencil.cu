@@ -87,10 +87,15 @@ __device__ __forceinline__ double2 ld_d2(const double* p) { return *reinterpret_
 __device__ __forceinline__ float4 neg_f4(float4 v) { return make_float4(-v.x, -v.y, -v.z, -v.w); }
 
 // Strip q (of nq in a row) and row j of this thread.  Blocks of 32 x 8 strips leave lanes
-// idle where a row is no multiple of 32 strips (48: a quarter, 16: half); there the
-// plane's strips are numbered through and a block takes 256 consecutive ones (flat): the
-// GS-RB solve of 192^3 2430 -> 2329 us, 64 uneven grids 50.9 -> 46.7 ms.  Other rows keep
-// the 32 x 8 block, which re-reads fewer neighbour rows.
+// idle where a row is no multiple of 32 strips (48: a quarter, 16: half); there a plane's
+// strips can be numbered through, 256 consecutive ones to a block (flat): the GS-RB solve
+// of 192^3 2430 -> 2329 us, 64 uneven grids 50.9 -> 46.7 ms.  The 32 x 8 block re-reads fewer
+// neighbour rows.  Rows of 16 to 255 strips, flat against 32 x 8: the update gains at every
+// ragged width (260 x 256 x 256, 49% idle, 125 against 165 us; 508, 0.8%, 235 against 247); the
+// restriction gains above a sixth of idle lanes (260: 37 against 45 us, 144^3: 10.2 against
+// 12.3) and loses below (320, a sixth, 51 against 47; 448: 59 against 55; 508: 66 against 59;
+// 112^3 and 224^3, an eighth: the same); the prolongation gains above it (260: 28 against 31;
+// 208, 19%: 18.8 against 16.8) and is the same below.
 __device__ __forceinline__ bool strip_at(int nq, int rows, int flat, int& q, int& j) {
     if (flat) {
         const int s = blockIdx.x * (BX * BY) + threadIdx.y * BX + threadIdx.x;
@@ -105,7 +110,10 @@ __device__ __forceinline__ bool strip_at(int nq, int rows, int flat, int& q, int
 struct StripGrid {
     int flat;
     long long gx, gy;
-    StripGrid(int nq, int rows) : flat(nq % BX != 0), gx((nq + BX - 1) / BX), gy((rows + BY - 1) / BY) {
+    // flat above 1 / `share` idle lanes (0: wherever there are any)
+    StripGrid(int nq, int rows, int share) : gx((nq + BX - 1) / BX), gy((rows + BY - 1) / BY) {
+        const long long lanes = BX * gx, idle = lanes - nq;
+        flat = share > 0 ? share * idle > lanes : idle > 0;
         if (flat) {
             gx = ((long long)nq * rows + BX * BY - 1) / (BX * BY);
             gy = 1;
@@ -2168,7 +2176,7 @@ cudaError_t launch_residual_restrict(const LevelGeom& g, const T* u, const T* rh
                                reinterpret_cast<uintptr_t>(coarse_out)) & 15) == 0;
         if (!has_faces(g) && (g.nx & 3) == 0 && (g.ny & 1) == 0 && (g.nz & 1) == 0 && aligned) {
             // as many blocks as the scalar launch at most (the partials buffer)
-            const StripGrid at(g.nx / 4, g.ny / 2);
+            const StripGrid at(g.nx / 4, g.ny / 2, 6);
             const long long gx = at.gx, gy = at.gy;
             const long long chunks = std::min<long long>(g.nz / 2, std::max(1LL, restrict_blocks(g) / (gx * gy)));
             int kc = (int)((g.nz + chunks - 1) / chunks);
@@ -2211,7 +2219,7 @@ cudaError_t launch_prolong_correct(const LevelGeom& g, const T* coarse, T* fine_
     if constexpr (std::is_same<T, float>::value) {
         const bool aligned = ((reinterpret_cast<uintptr_t>(coarse) | reinterpret_cast<uintptr_t>(fine_u)) & 15) == 0;
         if ((g.nx & 3) == 0 && (g.ny & 1) == 0 && (g.nz & 1) == 0 && aligned) {
-            const StripGrid at(g.nx / 4, g.ny / 2);
+            const StripGrid at(g.nx / 4, g.ny / 2, 6);
             const long long gx = at.gx, gy = at.gy;
             const long long chunks = std::min<long long>(g.nz / 2, std::max(1LL, 16LL * 152 / (gx * gy)));
             int kc = (int)((g.nz + chunks - 1) / chunks);
@@ -2236,7 +2244,7 @@ cudaError_t launch_update_residual(const LevelGeom& g, double* phi, const float*
                            reinterpret_cast<uintptr_t>(r64) | reinterpret_cast<uintptr_t>(r32)) & 15) == 0;
     if ((g.nx & 3) == 0 && aligned) {
         // (as many blocks as the scalar residual launch at most: the partials buffer)
-        const StripGrid at(g.nx / 4, g.ny);
+        const StripGrid at(g.nx / 4, g.ny, 0);
         const long long gx = at.gx, gy = at.gy;
         // z chunks that fill one wave of four blocks per SM, or up to three waves where
         // that leaves fewer slots idle: solves with one wave against as many blocks as
