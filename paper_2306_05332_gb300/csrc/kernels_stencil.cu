@@ -290,7 +290,7 @@ k_stage4(const LevelGeom g, const CoefT<float> cf, const float* __restrict__ ym1
 // relative (1.65e-16 with equal h), 1.76e-16 by k_stage's order.
 // 256^3, s = 3: the three stages took 468, 560 and 560 us by k_stage, 315, 413 and 447
 // us here, the FP64 pipe 83% busy.
-// V = 2: strips of two x cells (even nx, 16-byte aligned arrays).
+// V = 2: strips of two x cells (even nx, 16-byte aligned arrays; launch_stage64 says where).
 // ---------------------------------------------------------------------------
 struct Stage64 {
     double m1t;             // first stage: Y1 = c + m1t Z0
@@ -439,7 +439,12 @@ cudaError_t launch_stage64(const LevelGeom& g, int order, bool first, const Stag
                          reinterpret_cast<uintptr_t>(y0) | reinterpret_cast<uintptr_t>(z0) |
                          reinterpret_cast<uintptr_t>(rhs) | reinterpret_cast<uintptr_t>(out) |
                          reinterpret_cast<uintptr_t>(z0_out);
-    const bool two = (g.nx & 1) == 0 && (al & 15) == 0;
+    // Strips of two leave more lanes idle in narrow and ragged rows, and an FP64 instruction
+    // of a half-empty warp costs as much as one of a full warp: they are taken where they
+    // leave no more idle than single cells.  A stage by single cells and by strips of two:
+    // 32^3 4.5 and 6.5 us, 96^3 30 and 35, 160^3 120 and 129, 32 x 256 x 256 69 and 118; but
+    // 104^3 42 and 39, 128^3 62 and 58, 192^3 204 and 190 (64^3 12.2 and 12.5: the same).
+    const bool two = (g.nx & 1) == 0 && (al & 15) == 0 && g.nx > 64 && (g.nx + 63) / 64 * 2 == (g.nx + 31) / 32;
     const int bx = two ? 2 * BX : BX, kc = kchunk_for(g, bx, BY);
     const dim3 block(BX, BY, 1), grid((g.nx + bx - 1) / bx, (g.ny + BY - 1) / BY, (g.nz + kc - 1) / kc);
     if (two) launch_stage64_v<2>(order, first, faces, uniform, grid, block, st, g, cf, ym1, ym2, y0, z0, rhs, out, z0_out, kc);
