@@ -124,7 +124,8 @@ struct Here {
     int q, j, P, p0;                            // p0: first plane pair of the slab
     int row, plane;
     int o, oym, oyp, ozm, ozp, oxl, oxr;        // offsets in a buffer of the cells and of the strips around them
-    T sym, syp, szm, szp, sxl, sxr;             // -1 across a Dirichlet wall, else 1
+    int oys, oyn;                               // the y neighbours again: the one with sign sys and the other
+    T sym, syp, szm, szp, sxl, sxr, sys;        // -1 across a Dirichlet wall, else 1
     int to_lo, to_hi, lo_off, hi_off;           // CTA (-1: none) and offset of the ghost strips this thread feeds
     unsigned far_lo, far_hi;                    // their addresses in the cluster's shared memory (0: none) ...
     unsigned bar_lo, bar_hi;                    // ... and the barriers that their arrival counts on
@@ -182,6 +183,10 @@ __host__ __device__ __forceinline__ Here<T, TWOD> make_here(const TailParams<T>&
             if (!py) h.syp = T(-1);
         }
     }
+    const bool above = h.syp < T(0);            // (a row has one wall at most: ny >= 2)
+    h.oys = above ? h.oyp : h.oym;
+    h.oyn = above ? h.oym : h.oyp;
+    h.sys = above ? h.syp : h.sym;
     h.ozm = h.o - h.plane;
     h.ozp = h.o + 2 * h.plane;
     h.to_lo = h.to_hi = -1;
@@ -337,21 +342,30 @@ __global__ void __launch_bounds__(tail_threads<T>()) k_tail_levels(const __grid_
     auto ld = [](const T* a) { return *reinterpret_cast<const V*>(a); };
     auto st = [](T* a, V v) { *reinterpret_cast<V*>(a) = v; };
 
-    // L c - f of the thread's cells c from buffer y, nf = -f, by the second differences
-    // (lower - 2 c) + upper of each axis.  (Neighbours summed against one term
-    // -2 (h_x + h_y + h_z) c take two operations a cell less, but the rounding of that
-    // coefficient acts on c itself and not on its differences: one V-cycle of a smooth
-    // 48 x 64 x 56 field was off by 5.0 - 7.1e-7 with it, by 1.2 - 2.1e-7 level by level.)
+    // L c - f of the thread's cells c from buffer y, nf = -f, by the second differences of
+    // each axis: (lower - 2 c) + upper, in FP64, whose operations count, -2 c + (lower +
+    // upper), one fewer.  (Neighbours summed against one term -2 (h_x + h_y + h_z) c take
+    // another one or two less, but the rounding of that coefficient acts on c itself and not
+    // on its differences: one V-cycle of a smooth 48 x 64 x 56 field was off by
+    // 5.0 - 7.1e-7 with it, by 1.2 - 2.1e-7 level by level.)
     auto lap = [&](const H& h, const T* y, const V (&c)[2], const V (&nf)[2], V (&out)[2]) {
 #pragma unroll
         for (int a = 0; a < 2; ++a) {
             const int at = a * h.plane;
             const T xl = y[h.oxl + at], xr = y[h.oxr + at];
-            const V m2 = mul2(T(-2), c[a]);
-            const V dx = mk2(fmat(h.sxl, xl, m2.x) + c[a].y, fmat(h.sxr, xr, m2.y) + c[a].x);
-            const V dz = add2(a == 0 ? fma2(h.szm, ld(y + h.ozm), m2) : fma2(h.szp, ld(y + h.ozp), m2), c[1 - a]);
+            V dx, dz, dy;
+            if constexpr (sizeof(T) == 8) {
+                dx = fma2(T(-2), c[a], mk2(fmat(h.sxl, xl, c[a].y), fmat(h.sxr, xr, c[a].x)));
+                dz = fma2(T(-2), c[a], a == 0 ? fma2(h.szm, ld(y + h.ozm), c[1]) : fma2(h.szp, ld(y + h.ozp), c[0]));
+                if constexpr (!TWOD) dy = fma2(T(-2), c[a], fma2(h.sys, ld(y + h.oys + at), ld(y + h.oyn + at)));
+            } else {
+                const V m2 = mul2(T(-2), c[a]);
+                dx = mk2(fmat(h.sxl, xl, m2.x) + c[a].y, fmat(h.sxr, xr, m2.y) + c[a].x);
+                dz = add2(a == 0 ? fma2(h.szm, ld(y + h.ozm), m2) : fma2(h.szp, ld(y + h.ozp), m2), c[1 - a]);
+                if constexpr (!TWOD) dy = fma2(h.syp, ld(y + h.oyp + at), fma2(h.sym, ld(y + h.oym + at), m2));
+            }
             V v = fma2(h.hz, dz, nf[a]);
-            if constexpr (!TWOD) v = fma2(h.hy, fma2(h.syp, ld(y + h.oyp + at), fma2(h.sym, ld(y + h.oym + at), m2)), v);
+            if constexpr (!TWOD) v = fma2(h.hy, dy, v);
             out[a] = fma2(h.hx, dx, v);
         }
     };
