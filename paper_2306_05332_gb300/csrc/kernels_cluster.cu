@@ -939,7 +939,7 @@ bool tail_plan(TailParams<T>& p, bool twod, TailLaunch* out) {
         // smallest such
         const TailLevel<T>& L = p.lv[0];
         const long long cells = (long long)L.nx * L.ny * L.nz;
-        if (sizeof(T) == 8 && cells > kTailCells64) return false;
+        if (sizeof(T) == 8 && cells > (p.nl == 1 ? kTailCoarse64 : kTailCells64)) return false;
         const int np = L.nz / 2;
         if (cells > whole)
             for (int n = 2; n <= kTailMaxNC && n <= np; ++n)

@@ -280,9 +280,20 @@ cudaError_t coarse_configure();
 // ---- the coarse end of the V-cycle in one cluster launch (kernels_cluster.cu) --
 constexpr int kTailMaxS = 32;            // smoothing stages the coefficient table holds
 constexpr int kTailMaxLevels = 12;
-constexpr long long kTailWhole = 2560;   // cells of a level that every CTA holds whole (four a thread)
-constexpr long long kTailWhole64 = 64;   // the same in FP64: its arithmetic is worth splitting over more SMs
-constexpr long long kTailCells64 = 16384;    // FP64: cells up to which 16 SMs beat a launch per stage on all of them
+// Cells up to which every CTA holds a level whole (FP32: four a thread, all that fit).  Solves
+// with the line at 64, 512, 1024 and 2560: 24^3 814, 695, 695, 684 us, 32^3 1050, 941, 941, 941,
+// 256^2 1847, 1786, 1741, 1738.
+constexpr long long kTailWhole = 2560;
+// The same in FP64, whose arithmetic is worth splitting over more SMs: at 64, 512 and 2048 16^3
+// 2816, 2717, 2722 us, 24^3 2762, 2636, 3801, 256^2 5970, 5602, 5605.
+constexpr long long kTailWhole64 = 512;
+// FP64: cells of the first level up to which 16 SMs beat a launch per stage on all of them.
+// With 4096 cells on the cluster and not: 32^3 3518 and 3852 us; with 8000: 40^3 4517 and 3679,
+// 80^3 9930 and 8938; with 13824: 48^3 6327 and 4272, 96^3 13609 and 11524.
+constexpr long long kTailCells64 = 4096;
+// FP64, the coarsest level alone, whose other way is one SM: on the cluster and not, 22^3 cells
+// 5446 and 10216 us, 24^3 6.2 and 10.7 ms.  (28^3 and 32^3 would gain too: 10.5 -> 8.1 ms.)
+constexpr long long kTailCoarse64 = 16384;
 template <typename T>
 constexpr int tail_threads() {           // largest block, by the registers of a thread's cells
     return sizeof(T) == 8 ? 512 : 640;

@@ -44,7 +44,7 @@ def test_mixed(shape, levels, opts, want):
     assert _launches_per_cycle(shape, levels, "mixed", 0, **opts) > want
 
 
-@pytest.mark.parametrize("shape,levels,stages", [((64, 64, 64), 5, 2), ((48, 32, 40), 3, 1), ((16, 16, 16), 4, 1)])
+@pytest.mark.parametrize("shape,levels,stages", [((64, 64, 64), 5, 2), ((32, 32, 32), 4, 1), ((16, 16, 16), 4, 1)])
 def test_fp64(shape, levels, stages):
     # `stages` levels by nine stages, restriction and prolongation each; the launch, the
     # residual and the loop's step
