@@ -65,3 +65,35 @@ def test_thin_level():
         out[fused] = g.potential()
     assert _launches_per_cycle(shape, 0, "mixed", 1, coarse_tol=0.0, coarse_max_ss=3) == 0
     assert np.linalg.norm(out[1] - out[0]) < 1e-5 * np.linalg.norm(out[0])
+
+
+def test_resident_solves_from_several_threads():
+    # a grid and a stream per host thread; each solve's potential is what it is alone
+    import threading
+
+    import paper_2306_05332_gb300 as sg
+
+    shapes = [(32, 32, 32), (16, 24, 20), (128, 96), (16, 16, 16)]
+
+    def solve(i, out, barrier=None):
+        stream = torch.cuda.Stream()
+        make = sg.Grid if len(shapes[i]) == 3 else sg.Grid2D
+        g = make(shapes[i], precision="mixed", stream=stream.cuda_stream)
+        g.set_density(W.random_field(shapes[i], i), 1.0)
+        if barrier:
+            barrier.wait()
+        for _ in range(3):
+            g.solve(tol=1e-9)
+        out[i] = g.potential()
+
+    alone, together = {}, {}
+    for i in range(len(shapes)):
+        solve(i, alone)
+    barrier = threading.Barrier(len(shapes), timeout=60)
+    threads = [threading.Thread(target=solve, args=(i, together, barrier)) for i in range(len(shapes))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for i in range(len(shapes)):
+        np.testing.assert_array_equal(together[i], alone[i])
