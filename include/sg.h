@@ -110,7 +110,9 @@ typedef struct sg_options {
                                (a profiler that cannot see into graphs with
                                conditional nodes sees every kernel); 0: kernels
                                launched one by one                               [1]  */
-    int    fused;           /* fused multi-stage super-step kernels where possible  [1]  */
+    int    fused;           /* fused multi-stage super-step kernels, and one cluster
+                               launch for the coarse levels (both precisions and
+                               smoothers, 2D too), where possible               [1]  */
     int    smoother;        /* sg_smoother.  With SG_SMOOTH_GSRB one relaxation
                                (n_pre, n_post) is one red-black sweep, every cell
                                solving its own row (Dirichlet ghost folded into the
@@ -130,7 +132,9 @@ typedef struct sg_options {
     int    tile_rows;       /* rows of the tile of the fused s = 2, 3 super-step
                                with one stage per thread: 14 or 16; 0 = the kernel
                                with one column per thread, tiles by its launcher's
-                               cost model (faster; the same bits)             [0]  */
+                               cost model (faster; the same bits).  Heeded, as
+                               staging is, for a level's first super-step from zero
+                               and on levels of 2^22 cells and more           [0]  */
     int    inner_n_pre;     /* smoothing super-steps on the way down on levels
                                1 .. L-2; -1 = n_pre (the paper's N_pre on every
                                level)                                           [-1] */
@@ -401,9 +405,11 @@ sg_status sg_plan_sor_omega(int nx, int ny, int nz, const double lo[3], const do
  * the compulsory reads and writes of their input and output arrays, each cell
  * counted once, independent of caching.  While the profile is on, the cluster
  * launch that otherwise runs every coarse level that fits it (and, for small
- * grids, the whole solve) takes only the two coarsest levels, so that the other
- * classes are seen at every level; results agree to FP32 rounding of the inner
- * V-cycle.
+ * grids, the whole solve) takes only the two coarsest levels, and those only in
+ * a 3D mixed-precision RKL solve, where the coarsest has a multiple of four
+ * cells in x and the other at most 1024 in a plane.  So the other classes are
+ * seen at every level, but their shares are not those of an unprofiled solve;
+ * results agree to FP32 rounding of the inner V-cycle.
  * ------------------------------------------------------------------------ */
 #define SG_KERNEL_CLASSES 11
 typedef struct sg_kernel_stat {

@@ -13,7 +13,7 @@
 // size), and a level's V-cycle share at the default N_pre = 2, N_post = 1, s = 3 is
 // 13 launches.  Here a stage costs a chain of shared-memory loads and FMAs and a
 // barrier: 0.67 us on a 32^3 level over 16 CTAs, 0.25 us on 8^3 and below (a whole
-// 32^3 solve with the default options: 2.11 ms level by level, 0.81 ms resident).
+// 32^3 solve with the default options: 2.11 ms level by level, 0.79 ms resident).
 //
 // Cells.  A thread owns two cells of a row in two neighbouring planes (2 x 2 cells of a
 // two-dimensional level) through all stages: iterate, right-hand side, Y0, Z0 and

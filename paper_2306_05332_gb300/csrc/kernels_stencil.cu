@@ -289,7 +289,8 @@ k_stage4(const LevelGeom g, const CoefT<float> cf, const float* __restrict__ ym1
 // 80-bit arithmetic one RKL2 super-step of s = 3 on a smooth field is off by 1.3e-16
 // relative (1.65e-16 with equal h), 1.76e-16 by k_stage's order.
 // 256^3, s = 3: the three stages took 468, 560 and 560 us by k_stage, 315, 413 and 447
-// us here, the FP64 pipe 83% busy.
+// us here (311, 409, 442 under ncu, the FP64 pipe active 83% of the time; by operations
+// 0.77 of the rate that FMA chains reach).
 // V = 2: strips of two x cells (even nx, 16-byte aligned arrays; launch_stage64 says where).
 // ---------------------------------------------------------------------------
 struct Stage64 {

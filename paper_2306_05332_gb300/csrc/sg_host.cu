@@ -707,7 +707,9 @@ bool tail_params(const sg_grid* g, int L, int B, TailParams<W>& p, TailLaunch* t
 // 3.04 ms).  Level 0 joins only for the error equation (FP32, e = 0 at the start, no
 // face data).
 // While a profile is taken only the two coarsest levels are run by it, so that the
-// kernel classes of the others can be told apart.
+// kernel classes of the others can be told apart, and those within fixed limits: what a
+// profile reports of a grid (which class its coarse levels count in) does not move with
+// what fits the cluster.
 template <typename W>
 int tail_level(const sg_grid* g, int L, TailParams<W>& p, TailLaunch* t) {
     if (!g->opt.fused) return -1;
@@ -718,8 +720,8 @@ int tail_level(const sg_grid* g, int L, TailParams<W>& p, TailLaunch* t) {
             g->lv[L - 1].nx % 4 != 0 || (long long)g->lv[b].nx * g->lv[b].ny > 1024)
             return -1;
     }
-    // FP64: also the coarsest level alone (16^3: 0.70 ms a solve on one SM, whose FP64
-    // rate bounds it)
+    // FP64: also the coarsest level alone (one SM, the other way to run it, is bound by
+    // its FP64 rate: kTailCoarse64)
     for (; b <= (std::is_same<W, float>::value ? L - 2 : L - 1); ++b)
         if (tail_params<W>(g, L, b, p, t)) return b;
     return -1;

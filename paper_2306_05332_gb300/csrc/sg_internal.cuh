@@ -236,9 +236,9 @@ bool fused_supported(int order, int s);
 cudaError_t fused_configure();
 // out = Y_s of one super-step from y0 (nullptr: Y0 = 0) with homogeneous or
 // periodic ghosts; out must not alias y0.
-// tile_rows: 14 or 16 fixes the tile of the s = 2, 3 kernel; 0 lets its cost
-// model choose.  tma: that kernel stages planes by tensor-map box copies where
-// the level allows it (otherwise by per-strip copies).
+// s = 2, 3: tile_rows 0 without tma takes the kernel with one column per thread;
+// 14 or 16 the one with one stage per thread and tiles of so many rows, tma the
+// same with planes staged by tensor-map box copies where the level allows it.
 cudaError_t launch_superstep_fused(const LevelGeom& g, int order, int s, bool zero_y0, const FusedCoef& cf,
                                    const float* y0, const float* f, float* out, cudaStream_t st,
                                    int tile_rows = 0, bool tma = false);
