@@ -740,7 +740,7 @@ def run_ours(a, world, rank, local):
         torch.cuda.synchronize()
         ts = time.perf_counter() - t0
         # autotuned per size class: the smoother (order kept), s, tau, smoothing
-        # counts, fused on / off and the fused kernel's tile rows picked on the
+        # counts and fused on / off picked on the
         # first instance of each size, then given to every instance of that size
         tuned = {}
         for gb, pb, rb in zip(grids, probs, rhos):

@@ -317,7 +317,7 @@ typedef struct sg_tune_entry {
                                   rate: the coarse grid does not see it) */
     double ms_per_decade;      /* ms_per_cycle / -log10(factor): the score (lower is better) */
     int    n_pre, n_post;      /* smoothing super-steps per V-cycle tried */
-    int    tile_rows;          /* tile rows of the fused super-step tried (0: cost model) */
+    int    tile_rows;          /* the option of that name (0: one column per thread) */
     int    inner_n_pre, inner_n_post;   /* smoothing counts of levels 1 .. L-2 tried (-1: n_pre, n_post) */
 } sg_tune_entry;
 
